@@ -204,10 +204,9 @@ int gp_apply_pending_scale(gp_ctx *ctx);
  * must not outlive a cudaDeviceReset of that device.  The coefficient tables are written into
  * the array by a small kernel on cuda_stream (nothing is staged through host
  * memory).  All calls share the one array, which keeps the last call's
- * contents: calls whose work overlaps on the GPU race with each other.  The
- * x sweep (axis 0) runs one line per thread along contiguous x, so its
- * accesses are not coalesced and it is several times slower than the y and
- * z sweeps.  Errors: GP_EINVAL for bad arguments, GP_ECUDA if a CUDA call
+ * contents: calls whose work overlaps on the GPU race with each other.  An
+ * x sweep (axis 0) of many lines runs them two lanes each along contiguous x,
+ * uncoalesced, and is several times slower than the y and z sweeps.  Errors: GP_EINVAL for bad arguments, GP_ECUDA if a CUDA call
  * fails; the message is in gp_last_error(NULL).
  */
 int gp_sweep_noalloc(void *psi_device, const gp_grid *grid, int axis, double h,
@@ -279,14 +278,19 @@ int gp_slab_observables(gp_ctx *ctx, const double global_sums[9], gp_obs *out);
 
 /* Options of a context (gp_set_option / gp_get_option). */
 enum {
-    /* Sweep kernel: GP_PATH_AUTO picks per axis and mode; GP_PATH_EXACT is one
-     * line per thread with the elimination scratch in device memory;
-     * GP_PATH_TMA streams chunks of a tile of lines through shared memory with
+    /* Sweep kernel: GP_PATH_AUTO picks per axis and mode; GP_PATH_EXACT is a
+     * lane pair per line with the elimination scratch in device memory, or,
+     * for grids with too few lines to fill the GPU that way, each line in
+     * shared memory cut into pieces that many lanes solve at once, starting
+     * outside their pieces by a window whose truncation is below 2^-55
+     * (complex128) / 2^-40 (complex64); GP_PATH_TMA streams chunks of a tile of lines through shared memory with
      * TMA and back-substitutes over a window, which is only selected (and
      * only accepted) when a window W <= C (the chunk) has a truncation bound
      * max|c'|^(W+1) below 2^-40 (complex64) / 2^-55 (complex128): the
      * truncation repeats identically every step, so it is kept far below
-     * one rounding. */
+     * one rounding.  Under GP_PATH_AUTO a complex64 sweep reported as
+     * GP_PATH_TMA runs its arithmetic on the cut lines where that is faster
+     * (small grids); a request for GP_PATH_TMA streams. */
     GP_OPT_SWEEP_PATH = 1,
     /* Tile shape of the TMA sweep path: an index (0 .. GP_TILE_SHAPES - 1,
      * per precision) into the library's table of (lines per CTA, points per

@@ -525,6 +525,22 @@ int sweep_path(const gp_ctx *c, int axis)
     return c->prec == GP_C64 ? GP_PATH_TMA : GP_PATH_EXACT;
 }
 
+// Under GP_PATH_AUTO a complex64 sweep runs on the sub-line kernel where that
+// is faster than the TMA pipeline, which needs 128 lines for every CTA to
+// stream and walks each line row by row.  Measured on GB300 (us beyond a
+// launch; n rows a line, p points): TMA 8 + max(0.06 n, p / 370e3) on y and z,
+// 13 + max(0.125 n, p / 250e3) on x; sub-lines 4 + p / 210e3 and 7 + p / 150e3.
+// The lines cross between 128^3 (16 against 14 us on y, 36 against 23 on x)
+// and 256^3 (49 against 75, 72 against 117); 500 x 384 (2D): 31 against 8.
+bool prefers_split(const gp_ctx *c, int axis)
+{
+    if (c->prec != GP_C64 || c->path_opt != GP_PATH_AUTO || c->tile_shape != 0) return false;
+    if (sweep_path(c, axis) != GP_PATH_TMA) return false;
+    const double n = edge(c->grid, axis), p = (double)points(c->grid);
+    if (axis == 0) return 13.0 + std::max(0.125 * n, p / 250e3) > 7.0 + p / 150e3;
+    return 8.0 + std::max(0.06 * n, p / 370e3) > 4.0 + p / 210e3;
+}
+
 cudaError_t launch_sweep(gp_ctx *c, int axis, const gp::NonlinArgs *nl, bool nl_at_output,
                          const Partials *norm, int *blocks)
 {
@@ -550,17 +566,23 @@ cudaError_t launch_sweep(gp_ctx *c, int axis, const gp::NonlinArgs *nl, bool nl_
         return gp::launch_sweep_ff(c->tile_shape, c->mode, axis, c->maps[axis], c->ffax[c->mode][axis],
                                    g, nl ? &fn : nullptr, norm, c->err_dev, c->stream);
     }
+    gp::SplitPlan plan;
+    if (prefers_split(c, axis) && gp::split_plan(c->prec, ax, g, plan, true) &&
+        !(norm && c->mode == GP_REAL)) {
+        if (blocks) *blocks = gp::split_blocks(plan);
+        return gp::launch_sweep_split(plan, c->prec, c->mode, c->psi, ax, g, nl, nl_at_output, norm,
+                                      c->stream);
+    }
     if (sweep_path(c, axis) == GP_PATH_TMA) {
         if (blocks) *blocks = gp::tma_blocks(c->prec, c->tile_shape, g);
         return gp::launch_sweep_tma(c->prec, c->tile_shape, c->mode, axis, c->maps[axis], ax, g,
                                     nl, norm, c->err_dev, c->stream, nl_at_output);
     }
-    if (blocks) *blocks = gp::sweep_blocks(g);
     if (nl && !nl_at_output)
         return gp::launch_sweep_x(c->prec, c->mode, c->psi, c->work, ax, g, *nl, c->grid.ny,
                                   c->grid.nz, norm, c->stream);
     return gp::launch_sweep_yz(c->prec, c->mode, c->psi, c->work, ax, g, norm, c->stream,
-                               nl_at_output ? nl : nullptr);
+                               nl_at_output ? nl : nullptr, blocks);
 }
 
 bool modulated(const gp_ctx *c) { return c->g1 != 0.0; }

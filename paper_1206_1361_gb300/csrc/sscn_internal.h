@@ -187,13 +187,14 @@ cudaError_t launch_sweep_x(int prec, int mode, void *psi, void *work,
                            const AxisTables &ax, const SweepGeom &g,
                            const NonlinArgs &nl, int ny, int nz,
                            const Partials *norm_out, cudaStream_t st);
-// y or z sweep; norm_out != nullptr adds the FP64 sum |u|^2 per block;
+// y or z sweep; norm_out != nullptr adds the FP64 sum |u|^2 per block (their
+// number to *blocks, if not null);
 // nlout != nullptr (real time, no norm) applies calcnu to every result
 // before it is stored, with the tables in this sweep's order.
 cudaError_t launch_sweep_yz(int prec, int mode, void *psi, void *work,
                             const AxisTables &ax, const SweepGeom &g,
                             const Partials *norm_out, cudaStream_t st,
-                            const NonlinArgs *nlout = nullptr);
+                            const NonlinArgs *nlout = nullptr, int *blocks = nullptr);
 // calcnu as its own pass over every point (x lines; tables in x, y, z order)
 // with the FP64 sums |psi|^2 into `blocks` partials: the imaginary-time
 // symmetric splitting's second half step, after the renormalisation.
@@ -207,7 +208,31 @@ cudaError_t launch_build_pot3(void *p3, const double2 *px, const double2 *py, co
 // Device step counter (modulated g): set it, or add one.
 cudaError_t launch_set_step(long long *step, long long value, cudaStream_t st);
 cudaError_t launch_add_step(long long *step, cudaStream_t st);
+// Most norm partials (blocks) any of these sweeps writes for this geometry.
 int sweep_blocks(const SweepGeom &g);
+
+// ---- sub-line sweeps (sscn_split.cu) ----------------------------------------
+// Launch shape of a sweep whose lines are solved by 2 S lanes of at most P rows
+// each (FP64: S sub-lines eliminated from both ends by a lane pair), with
+// windows of W rows.
+struct SplitPlan {
+    int P = 0, S = 0, W = 0;
+    bool x = false;              // lines contiguous in memory
+    bool increment = false;      // complex64: the TMA path's arithmetic, else the exact path's
+    int per = 0, threads = 0;    // lines per block, threads per block
+    unsigned grid_x = 0, grid_y = 0;
+    size_t smem = 0;
+};
+// Whether the sweep of these lines runs that way, and how.
+bool split_plan(int prec, const AxisTables &ax, const SweepGeom &g, SplitPlan &plan,
+                bool increment = false);
+int split_blocks(const SplitPlan &plan);
+int split_most_blocks(const SweepGeom &g);
+// nl: calcnu on every loaded point (x), or with nl_at_output on every result
+// (real time, y / z); norm_out (imaginary time, y / z): as launch_sweep_yz.
+cudaError_t launch_sweep_split(const SplitPlan &plan, int prec, int mode, void *psi,
+                               const AxisTables &ax, const SweepGeom &g, const NonlinArgs *nl,
+                               bool nl_at_output, const Partials *norm_out, cudaStream_t st);
 
 // scale <- 1 / sqrt(w * sum(partials)); flags a non-finite or non-positive sum.
 cudaError_t launch_norm_finish(const double *partials, int count, double w,

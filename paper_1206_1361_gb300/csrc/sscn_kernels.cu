@@ -618,7 +618,9 @@ int point_blocks(long long count)
 
 int sweep_blocks(const SweepGeom &g)
 {
-    return ((g.lines_a + kLinesPerBlock - 1) / kLinesPerBlock) * g.lines_b;
+    const int pairs = ((g.lines_a + kLinesPerBlock - 1) / kLinesPerBlock) * g.lines_b;
+    const int split = split_most_blocks(g);
+    return pairs > split ? pairs : split;
 }
 
 cudaError_t launch_sweep_x(int prec, int mode, void *psi, void *work,
@@ -626,6 +628,9 @@ cudaError_t launch_sweep_x(int prec, int mode, void *psi, void *work,
                            const NonlinArgs &nl, int, int, const Partials *norm_out,
                            cudaStream_t st)
 {
+    SplitPlan plan;
+    if (!norm_out && split_plan(prec, ax, g, plan))
+        return launch_sweep_split(plan, prec, mode, psi, ax, g, &nl, false, nullptr, st);
     if (nl.p3) {
         // the precomputed potential factors: FP64 real time, no norm partials
         if (prec != kC128 || mode != 1 || norm_out) return cudaErrorInvalidValue;
@@ -637,8 +642,15 @@ cudaError_t launch_sweep_x(int prec, int mode, void *psi, void *work,
 
 cudaError_t launch_sweep_yz(int prec, int mode, void *psi, void *work,
                             const AxisTables &ax, const SweepGeom &g,
-                            const Partials *norm_out, cudaStream_t st, const NonlinArgs *nlout)
+                            const Partials *norm_out, cudaStream_t st, const NonlinArgs *nlout,
+                            int *blocks)
 {
+    SplitPlan plan;
+    if (!(norm_out && (mode == 1 || g.pstride == 1)) && split_plan(prec, ax, g, plan)) {
+        if (blocks) *blocks = split_blocks(plan);
+        return launch_sweep_split(plan, prec, mode, psi, ax, g, nlout, nlout != nullptr, norm_out, st);
+    }
+    if (blocks) *blocks = ((g.lines_a + kLinesPerBlock - 1) / kLinesPerBlock) * g.lines_b;
     if (nlout) {
         // the symmetric splitting's second half step, fused where the real-time
         // last sweep stores (imaginary time takes a separate pass after the

@@ -1,0 +1,115 @@
+"""Sub-line sweeps (sscn_split.cu): grids whose lines are cut into pieces that
+many lanes solve.  Shapes put every remainder of that cut on some axis (one
+row, one row more or less than full pieces, a single piece), uneven tiles of
+neighbouring lines, and lines longer than a block of 8 rows a lane holds.
+
+Tolerances.  FP64 against the oracle: 1e-12 of the norm (a few hundred
+roundings of 2^-53).  complex64 sweeps alone (no trap, g = 0) against the
+oracle: 4 roundings of 2^-23 per sweep set.  complex64 against the TMA sweeps
+it stands in for, whose arithmetic it keeps: one rounding, 2^-24."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1206_1361_gb300 import gp
+from tests.gpu_util import oracle_params, rel_l2, require_gpu
+
+W3 = (1.0, 1.5, 2.0)
+# n - 1 = 16 k, 16 k + 1, 32 k + 1, one piece, 2 and 3 rows
+SHAPES = [(17, 33, 18), (34, 16, 3), (49, 35, 66), (200, 7, 140), (131, 3, 4), (500, 129, 1),
+          (3, 1100, 1), (4100, 5, 1), (33, 2051, 1)]
+
+
+def rand_state(shape, seed):
+    nx, ny, nz = shape
+    rng = np.random.default_rng(seed)
+    a = rng.standard_normal((nz, ny, nx)) + 1j * rng.standard_normal((nz, ny, nx))
+    a[:, :, 0] = a[:, 0, :] = 0
+    if nz > 1:
+        a[0] = 0
+    return a * 0.3
+
+
+def spacing(shape, kappa, dt):
+    h = (dt / (4.0 * kappa)) ** 0.5
+    return (h, 1.1 * h, 1.25 * h if shape[2] > 1 else 1.0)
+
+
+def trap_of(shape):
+    return W3 if shape[2] > 1 else (1.0, 1.5, 0.0)
+
+
+def run(shape, h, dt, w, g, mode, prec, steps, psi0, path=gp.GP_PATH_AUTO):
+    with gp.Solver(shape, h, dt, *w, g, mode, prec) as s:
+        s.set_path(path)
+        s.load(psi0.astype(s.dtype)).step(steps)
+        return s.psi().astype(np.complex128)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("mode", [gp.GP_IMAG, gp.GP_REAL])
+@pytest.mark.parametrize("kappa", [0.0125, 0.05, 0.4])
+def test_fp64_matches_the_oracle(shape, mode, kappa):
+    require_gpu()
+    dt, g, steps, w = 1e-3, 4.0, 3, trap_of(shape)
+    h = spacing(shape, kappa, dt)
+    psi0 = rand_state(shape, 7)
+    got = run(shape, h, dt, w, g, mode, gp.GP_C128, steps, psi0)
+    want = psi0.copy()
+    oracle.step(oracle_params(shape, h, dt, w, g, mode), want, steps)
+    assert rel_l2(got, want) <= 1e-12
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("mode", [gp.GP_IMAG, gp.GP_REAL])
+@pytest.mark.parametrize("kappa", [0.0125, 0.05, 0.4])
+@pytest.mark.parametrize("path", [gp.GP_PATH_AUTO, gp.GP_PATH_EXACT])
+def test_complex64_sweeps_match_the_oracle(shape, mode, kappa, path):
+    require_gpu()
+    dt, steps = 1e-3, 3
+    h = spacing(shape, kappa, dt)
+    psi0 = rand_state(shape, 8).astype(np.complex64)
+    got = run(shape, h, dt, (0.0, 0.0, 0.0), 0.0, mode, gp.GP_C64, steps, psi0, path)
+    want = psi0.astype(np.complex128)
+    oracle.step(oracle_params(shape, h, dt, (0.0, 0.0, 0.0), 0.0, mode), want, steps)
+    assert rel_l2(got, want) <= steps * 4 * 2.0 ** -23
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("shape", [(18, 33, 17), (200, 7, 140), (500, 129, 1), (66, 1025, 1), (4, 3, 35)])
+@pytest.mark.parametrize("mode", [gp.GP_IMAG, gp.GP_REAL])
+@pytest.mark.parametrize("strang", [False, True])
+def test_complex64_keeps_the_tma_sweeps_arithmetic(shape, mode, strang):
+    require_gpu()
+    dt, w = 1e-3, trap_of(shape)
+    h = spacing(shape, 0.02, dt)
+    psi0 = rand_state(shape, 5)
+    got = []
+    for path in (gp.GP_PATH_AUTO, gp.GP_PATH_TMA):
+        with gp.Solver(shape, h, dt, *w, 4.0, mode, gp.GP_C64) as s:
+            s.set_path(path).set_splitting(gp.GP_SPLIT_STRANG if strang else gp.GP_SPLIT_LIE)
+            s.load(psi0.astype(np.complex64)).step(4)
+            got.append(s.psi().astype(np.complex128))
+    assert rel_l2(got[0], got[1]) <= 2.0 ** -24
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("mode", [gp.GP_IMAG, gp.GP_REAL])
+@pytest.mark.parametrize("prec", [gp.GP_C128, gp.GP_C64])
+@pytest.mark.parametrize("table", [0, 1])
+@pytest.mark.parametrize("shape", [(49, 35, 18), (130, 67, 1)])
+def test_symmetric_splitting_and_modulated_g(mode, prec, table, shape):
+    require_gpu()
+    dt, g, g1, omega, steps = 2e-3, 6.0, 4.0, 25.0, 12
+    h = spacing(shape, 0.03, dt)
+    psi0 = rand_state(shape, 9)
+    w = trap_of(shape)
+    with gp.Solver(shape, h, dt, *w, g, mode, prec) as s:
+        gp.gp_set_option(s.ctx, gp.GP_OPT_POTENTIAL_TABLE, table)
+        s.set_splitting(gp.GP_SPLIT_STRANG).set_modulation(g1, omega)
+        s.load(psi0.astype(s.dtype)).step(steps)
+        got = s.psi().astype(np.complex128)
+    want = oracle.step_ext(oracle_params(shape, h, dt, w, g, mode), psi0.copy(), steps, 0, True, g1, omega)
+    assert rel_l2(got, want) <= (1e-12 if prec == gp.GP_C128 else steps * 4 * 2.0 ** -23)
