@@ -1,0 +1,550 @@
+// sscn_inc.cu -- Crank-Nicolson sweeps (calclux, calcluy, calcluz, calcnu
+// fused) of a complex128 psi whose increment is computed on the FP32 pipe.
+//
+// What bounds the FP64 sweeps.  GB300 issues a warp-wide FP64 instruction every
+// 64 clocks per quarter-SM against 2 for a packed FP32 one; a sweep's 12 (real
+// time) or 6 - 8 (imaginary time) FP64 instructions a point, 28 with calcnu,
+// hold it at a seventh of the HBM bandwidth.
+//
+// Here psi stays FP64, but the sweep computes the increment 2 Delta of
+//     (I - kappa L) Delta = kappa L psi,   u = psi + 2 Delta,
+// in float-float arithmetic (sscn_ff.cuh, ~48 significant bits) and adds it to
+// the FP64 psi: 2 FP64 instructions a point.  |2 Delta| is at most 8 kappa
+// max|psi| and about kappa (k h)^2 |psi| on a smooth state, so with kappa up to
+// kIncKappaReal / kIncKappaImag the rounding of the increment stays at or below
+// that of the FP64 form u = 2 v - psi, which rounds at full size several times.
+// calcnu likewise: the nonlinear factor's distance from 1 is computed in
+// float-float, the potential factor multiplies in FP64.
+//
+// Measured (GB300, 256^3 real time, kappa = 0.0125): y and z sweeps 392 -> 226
+// us, x with calcnu 889 -> 432 us (8 FP64 instructions a point there: 230 us of
+// the FP64 pipe); the y sweep issues about 250 instructions a point, half of
+// them integer conversions and addresses, 56 % of the issue slots.  Relative L2
+// error against FP64 truth, start and here: 64^3 imaginary, 100 steps, 5.3e-15
+// and 2.1e-15; 256^3 real, 10 steps, 6.8e-15 and 4.4e-15; 128 x 96 x 80 real at
+// kappa = 0.05, 20 steps, 1.5e-14 and 6.6e-15.  In imaginary time the state
+// hardly changes from step to step and the rounding of the lifted psi repeats:
+// at kappa = 0.05 (500 x 384, 40 steps) 2.4e-15 against 1.6e-15, hence the
+// smaller kIncKappaImag.
+//
+// The lines are cut and solved as in sscn_split.cu (half sub-lines of at most P
+// rows, whole lines in shared memory).  Per row, r_j = kappa mult_j:
+//     s_j = psi_{j-1} - 2 psi_j + psi_{j+1}
+//     e_j = s_j + r_{j-1} e_{j-1}              forward, from either end
+//     g_k = kappa mid_k (s_k + r e_{k-1} + r e_{k+1}),  2 Delta_k = 2 g_k
+//     g_j = r_j (e_j + g_{j+1}),               2 Delta_j = 2 g_j
+// (Delta = kappa D with (I - kappa L) D = s): the product that carries the back
+// substitution to the next row is the increment itself.  A window's rows
+// further than `near` rows from the lane's own, whose carry is damped below
+// 2^-26 on the way, run in plain FP32.
+//
+// Conversions go through the bits of the double with integer instructions (the
+// FP64 <-> FP32 conversion instructions run on the FP64 pipe).  Values enter
+// multiplied by 2^kLift, which puts the full float-float precision at 2^-105
+// .. 2^93; a block that holds anything larger, or not finite, sweeps in FP64.
+
+#include "sscn_ff.cuh"
+#include "sscn_split.cuh"
+
+namespace gp {
+
+using namespace gp::sp;
+using gp::ff::f2;
+using FC = gp::ff::C;
+
+namespace {
+
+constexpr int kIncP = 8;                 // rows a lane
+constexpr double kIncKappaReal = 0.06, kIncKappaImag = 0.025;
+constexpr int kLift = 30;
+constexpr int kIncEnds = 2 * kSplitEnds + 1;
+
+struct IncArgs {
+    SplitArgs<double> s;
+    int near;                            // window rows in float-float
+    FfCoef rinf;                         // r past conv
+    FfCoef kmid[kIncEnds];               // kappa mid_k
+};
+
+// ------------------------------------------------------------- conversions
+
+constexpr unsigned kOff = (unsigned)(1023 - 127 - kLift) << 20;   // FP64 - FP32 exponent, lifted
+
+// Not finite, or too large for a lifted float.
+__device__ __forceinline__ bool too_large(double x)
+{
+    return ((unsigned)__double2hiint(x) & 0x7fffffffu) >= kOff + (250u << 20);
+}
+
+// 2^kLift x as a float-float pair: hi the nearest float (ties away from zero),
+// lo the float nearest the rest.  With x = s m 2^(e-52), m the 53-bit
+// significand: hi = s r 2^(e-23), r = (m + 2^28) >> 29, and x - hi = s d
+// 2^(e-52), d = m - 2^29 r = ((m + 2^28) mod 2^29) - 2^28.
+__device__ __forceinline__ float2 lift(double x)
+{
+    const unsigned L = (unsigned)__double2loint(x), H = (unsigned)__double2hiint(x);
+    const unsigned L2 = L + 0x10000000u, E = H - kOff, E2 = E + (L2 < L ? 1u : 0u);
+    const unsigned sign = H & 0x80000000u, mag = H & 0x7fffffffu;
+    float hi = __uint_as_float((__funnelshift_l(L2, E2, 3) & 0x7fffffffu) | sign);
+    const int d = (int)(L2 & 0x1fffffffu) - 0x10000000;
+    const float ulp = __uint_as_float((((E - (52u << 20)) << 3) & 0x7f800000u) | sign);   // s 2^(e-52)
+    float lo = __int2float_rn(d) * ulp;
+    if (mag < kOff + (53u << 20)) lo = 0.f;
+    if (mag < kOff + (1u << 20)) hi = 0.f;
+    return f2(hi, lo);
+}
+
+// 2^TIMES x (SCALED: x lifted) as FP64: exact, zero for zero.
+template <int TIMES, bool SCALED> __device__ __forceinline__ double widen(float x)
+{
+    constexpr unsigned off = (SCALED ? kOff : (unsigned)(1023 - 127) << 20) + ((unsigned)TIMES << 20);
+    const unsigned f = __float_as_uint(x), mag = f & 0x7fffffffu;
+    const unsigned H = mag == 0u ? 0u : (mag >> 3) + off;
+    return __hiloint2double((int)(H | (f & 0x80000000u)), (int)(f << 29));
+}
+
+// 2^(TIMES - kLift) (hi + lo) as FP64 with one FP64 addition; or (MERGE) with
+// none: hi's bits as FP64 bits plus lo, renormalised to at most half an ulp of
+// hi, in units of FP64's last place (carries and borrows run through the
+// exponent field as they should; below a power of two the place is half as
+// large).  MERGE takes about 12 more instructions: for the x sweep, which the
+// FP64 pipe bounds.
+template <int TIMES, bool SCALED, bool MERGE> __device__ __forceinline__ double drop(float h, float l)
+{
+    if (!MERGE) return widen<TIMES, SCALED>(h) + widen<TIMES, SCALED>(l);
+    const float2 z = ff::s_two_sum(h, l);
+    const unsigned f = __float_as_uint(z.x), ef = f & 0x7f800000u;
+    const float units = __uint_as_float(ef >= (53u << 23) ? (306u << 23) - ef : 0u);      // 2^(52 - e)
+    int li = __float2int_rn(z.y * units);
+    const int neg = (int)f >> 31;
+    li = (li ^ neg) - neg;
+    if ((f & 0x7fffffu) == 0u && li < 0) li *= 2;
+    const long long b = __double_as_longlong(widen<TIMES, SCALED>(z.x)) + (long long)li;
+    return ef == 0u ? 0.0 : __longlong_as_double(b);
+}
+
+__device__ __forceinline__ FC lift(double2 p)
+{
+    const float2 x = lift(p.x), y = lift(p.y);
+    return FC{f2(x.x, y.x), f2(x.y, y.y)};
+}
+
+// p + 2^(TIMES - kLift) z
+template <int TIMES, bool MERGE> __device__ __forceinline__ double2 plus(double2 p, FC z)
+{
+    return make_double2(p.x + drop<TIMES, true, MERGE>(z.hi.x, z.lo.x),
+                        p.y + drop<TIMES, true, MERGE>(z.hi.y, z.lo.y));
+}
+
+__device__ __forceinline__ float4 pack(FC z) { return make_float4(z.hi.x, z.hi.y, z.lo.x, z.lo.y); }
+__device__ __forceinline__ FC unpack(float4 v) { return FC{f2(v.x, v.y), f2(v.z, v.w)}; }
+
+// ------------------------------------------------------------------ calcnu
+
+// G 2^(-2 kLift) as a pair: times |lift(p)|^2 it gives a = G |p|^2.
+__device__ __forceinline__ float2 lifted_g(double G)
+{
+    const double g = ldexp(G, -2 * kLift);
+    const float h = (float)g;
+    return f2(h, (float)(g - (double)h));
+}
+
+// Real time: exp(-i a) p, a = G |p|^2, as p + (exp(-i a) - 1) p with the factor
+// from its Taylor series in float-float for |a| < 2^-8 (first dropped terms
+// a^6 / 720 and a^7 / 5040 below 2^-57), in FP64 beyond.
+__device__ __forceinline__ double2 nonlinear_real(double2 p, float2 g, double G)
+{
+    const FC z = lift(p);
+    const float2 a = ff::s_mul(g, ff::abs2(z));
+    if (fabsf(a.x) < 0x1p-8f && !too_large(p.x) && !too_large(p.y)) {
+        const float q = __fmul_rn(a.x, a.x);
+        float qe = fmaf(a.x, a.x, -q);
+        qe = fmaf(2.f * a.x, a.y, qe);
+        const float2 dr = f2(-0.5f * q, fmaf(q * q, 1.f / 24, -0.5f * qe));
+        const float2 di = f2(-a.x, fmaf(a.x * q, fmaf(q, -1.f / 120, 1.f / 6), -a.y));
+        const FfCoef D{f2(dr.x, dr.x), f2(dr.y, dr.y), f2(-di.x, di.x), f2(-di.y, di.y)};
+        return plus<0, true>(p, ff::cmul(z, D));
+    }
+    double cs, sn;
+    expmi_small(G * fma(p.x, p.x, p.y * p.y), cs, sn);
+    return make_double2(fma(cs, p.x, sn * p.y), fma(cs, p.y, -sn * p.x));
+}
+
+// Imaginary time: f exp(-a), a = G |p|^2, as f + f (exp(-a) - 1) likewise.
+__device__ __forceinline__ double factor_imag(double2 p, double f, float2 g, double G)
+{
+    const float2 a = ff::s_mul(g, ff::abs2(lift(p)));
+    if (fabsf(a.x) < 0x1p-8f && !too_large(p.x) && !too_large(p.y)) {
+        const float q = __fmul_rn(a.x, a.x);
+        float qe = fmaf(a.x, a.x, -q);
+        qe = fmaf(2.f * a.x, a.y, qe);
+        const float2 s = ff::s_two_sum(-a.x, 0.5f * q);
+        const float tail = fmaf(q, fmaf(a.x, -1.f / 120, 1.f / 24) * q, -a.x * q * (1.f / 6));
+        const float2 eps = ff::s_norm(f2(s.x, s.y + ((0.5f * qe - a.y) + tail)));
+        return fma(f, drop<0, false, true>(eps.x, eps.y), f);
+    }
+    return f * expm_small(G * fma(p.x, p.x, p.y * p.y));
+}
+
+// calcnu at stored point i (MODE 0: c.pyz carries the pending scale).
+template <int MODE, bool P3>
+__device__ __forceinline__ double2 calcnu_at(double2 p, const Calcnu<double, MODE> &c, int i, double2 p3, float2 g,
+                                             double G)
+{
+    if (MODE == 0) {
+        const double f = factor_imag(p, c.pyz.x * c.px[i].x, g, G);
+        return make_double2(p.x * f, p.y * f);
+    }
+    const double2 w = nonlinear_real(p, g, G);
+    return P3 ? cmulc(w, p3) : cmulc(cmulc(w, c.pyz), c.px[i]);
+}
+
+// ------------------------------------------------------------------- solve
+
+// r_t for t = -1 .. conv and the middle rows' kappa mid_k in shared memory.
+__host__ __device__ __forceinline__ size_t inc_coef_bytes(int conv) { return (size_t)(conv + 2 + kIncEnds) * sizeof(FfCoef); }
+
+template <int MODE> __device__ __forceinline__ void stage_inc(const IncArgs &A, void *to)
+{
+    FfCoef *tab = static_cast<FfCoef *>(to);
+    const int len = A.s.conv + 2;
+    for (int q = threadIdx.x; q < len; q += blockDim.x) {
+        FfCoef r = A.rinf;
+        if (q == 0) r = ff::expand(0.0, 0.0);
+        else if (q <= A.s.conv) {
+            const double2 v = ktimes<double, MODE>(A.s.k, A.s.mult[q - 1]);
+            r = ff::expand(v.x, v.y);
+        }
+        tab[q] = r;
+    }
+    for (int q = threadIdx.x; q < kIncEnds; q += blockDim.x) tab[len + q] = A.kmid[q];
+}
+
+// z r: kappa-scaled coefficients are real in imaginary time
+template <int MODE> __device__ __forceinline__ FC rtimes(FC z, const FfCoef &r)
+{
+    return MODE == 0 ? ff::rmul(z, r) : ff::cmul(z, r);
+}
+
+template <int MODE> struct IncLane : HalfLine {
+    const IncArgs &A;
+    const FfCoef *tab;       // stage_inc
+
+    __device__ __forceinline__ IncLane(const IncArgs &args, const void *tables, int seg)
+        : HalfLine(args.s.n, args.s.S, args.s.W, seg), A(args), tab(static_cast<const FfCoef *>(tables))
+    {
+    }
+    __device__ __forceinline__ const FfCoef &r(int t) const { return tab[min(t, A.s.conv) + 1]; }
+
+    // Solve.  ld(i): lifted psi at row i (0 at rows 0 and n); out(q, i, g): the
+    // row's g (lifted), q its place among the lane's rows (0 .. P -
+    // 1 from `first`).  SYNC: a block barrier between the last ld and the first
+    // out.  Every thread of the block calls this; `active` marks lanes with a
+    // line, pair is the lane distance of a sub-line's halves.
+    template <bool SYNC, typename Ld, typename Out>
+    __device__ __forceinline__ void solve(bool active, int pair, Ld ld, Out out) const
+    {
+        FC e = ff::cz(), ev[kIncP], cur = ff::cz(), d0 = ff::cz();
+        if (active) {
+            int t = ts;
+            const int t1 = max(ts, to - A.near);
+            if (t < t1) {
+                // far rows of the window in FP32
+                float2 ee = f2(0.f, 0.f);
+                const FC a0 = ld(row(t - 1));
+                FC a1 = ld(row(t));
+                float2 dd = ff::add(ff::sub(a1.hi, a0.hi), ff::sub(a1.lo, a0.lo));
+                for (; t < t1; ++t) {
+                    const FC a2 = ld(row(t + 1));
+                    const float2 dn = ff::add(ff::sub(a2.hi, a1.hi), ff::sub(a2.lo, a1.lo));
+                    const FfCoef &k = r(t - 1);
+                    float2 s = ff::sub(dn, dd);
+                    s = ff::fma2(ee, k.rh, s);
+                    if (MODE != 0) s = ff::fma2(ff::swap(ee), k.ih, s);
+                    ee = s;
+                    dd = dn;
+                    a1 = a2;
+                }
+                e.hi = ee;
+            }
+            cur = ld(row(t));
+            d0 = ff::sub(cur, ld(row(t - 1)));
+            auto rhs = [&](int at) {
+                const FC next = ld(row(at + 1)), d1 = ff::sub(next, cur), s = ff::sub(d1, d0);
+                cur = next;
+                d0 = d1;
+                return s;
+            };
+            for (; t < to; ++t) e = ff::add(rhs(t), rtimes<MODE>(e, r(t - 1)));
+            // (coefficients from shared memory for every lane: a separate path
+            // with the constants in registers made the warps that hold a line's
+            // end run both)
+#pragma unroll
+            for (int q = 0; q < kIncP; ++q)
+                if (to + q <= te) ev[q] = e = ff::add(rhs(to + q), rtimes<MODE>(e, r(to + q - 1)));
+        }
+        // the carries of both halves meet in the middle row
+        const FC c = rtimes<MODE>(e, r(te));
+        FC o;
+        o.hi.x = __shfl_xor_sync(0xffffffffu, c.hi.x, pair);
+        o.hi.y = __shfl_xor_sync(0xffffffffu, c.hi.y, pair);
+        o.lo.x = __shfl_xor_sync(0xffffffffu, c.lo.x, pair);
+        o.lo.y = __shfl_xor_sync(0xffffffffu, c.lo.y, pair);
+        FC g = ff::cz();
+        if (active && top) {
+            const FC next = ld(row(kt + 1)), s = ff::sub(ff::sub(next, cur), d0);
+            g = rtimes<MODE>(ff::add(ff::add(s, c), o), tab[A.s.conv + 2 + mid_at(A.s.S)]);
+        }
+        if (SYNC) __syncthreads();
+        if (active && top) out(kt - to, row(kt), g);
+        FC w;
+        w.hi.x = __shfl_xor_sync(0xffffffffu, g.hi.x, pair);
+        w.hi.y = __shfl_xor_sync(0xffffffffu, g.hi.y, pair);
+        w.lo.x = __shfl_xor_sync(0xffffffffu, g.lo.x, pair);
+        w.lo.y = __shfl_xor_sync(0xffffffffu, g.lo.y, pair);
+        if (!top) g = w;
+        if (active) {
+#pragma unroll
+            for (int q = kIncP - 1; q >= 0; --q)
+                if (to + q <= te) {
+                    g = rtimes<MODE>(ff::add(ev[q], g), r(to + q));
+                    out(q, row(to + q), g);
+                }
+        }
+    }
+};
+
+// ----------------------------------------------------------------- kernels
+
+// Resident blocks the kernels are compiled for: 3 of 256 threads (80 registers
+// a thread).
+template <int THREADS> constexpr int kMinBlocks = THREADS == 256 ? 3 : 1;
+
+// x sweep: as k_split_x, thread (row, seg) moving the row's points seg, seg + 2 S,
+// ...  A point's calcnu goes back to memory and is read again (from L1 or L2)
+// when its increment is there: kept in registers, it cost a third of the
+// resident warps.
+template <int MODE, bool NL, bool P3, int THREADS>
+__global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_x(const __grid_constant__ IncArgs A)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ double g_of_step;
+    __shared__ float2 g_lifted;
+    const SplitArgs<double> &a = A.s;
+    const int n = a.n, pitch = slot_of(n) + 1;
+    unsigned char *coef = smem_raw, *coef64 = coef + inc_coef_bytes(a.conv);
+    Calcnu<double, MODE> *row_nl = reinterpret_cast<Calcnu<double, MODE> *>(coef64 + coef_bytes<double>(a.conv));
+    float4 *tile = reinterpret_cast<float4 *>(row_nl + a.per);
+    const int line0 = blockIdx.x * a.per;
+    const int rows = min(a.per, a.lines_a * a.lines_b - line0);
+    const int lanes = 2 * a.S;
+    const int q = threadIdx.x / lanes, seg = threadIdx.x - q * lanes;
+    const bool active = q < rows;
+    const int at = (active ? q : 0) * pitch;
+    double2 *row = a.psi + (long long)(line0 + (active ? q : 0)) * n;
+    double2 v[kIncP], f3[NL && P3 ? kIncP : 1];
+    if (active) {
+#pragma unroll
+        for (int b = 0; b < kIncP; ++b) {
+            const int i = 1 + seg + b * lanes;
+            if (i < n) {
+                v[b] = row[i];
+                if constexpr (NL && P3) f3[b] = a.p3[(long long)(line0 + q) * n + i];
+            }
+        }
+    }
+    if (NL && threadIdx.x == 0) {
+        const double G = a.sg.value(), sc = MODE == 0 && a.scale ? *a.scale : 1.0;
+        g_of_step = G * sc * sc;
+        g_lifted = lifted_g(G * sc * sc);
+    }
+    if (NL && !P3)
+        for (int r = threadIdx.x; r < rows; r += blockDim.x) {
+            const int L = line0 + r;
+            row_nl[r].setup(a.px, a.py, a.pz, nullptr, nullptr, nullptr, L % a.lines_a, L / a.lines_a, 0.0, a.scale);
+        }
+    stage_inc<MODE>(A, coef);
+    for (int r = threadIdx.x; r < a.per; r += blockDim.x)
+        tile[r * pitch] = tile[r * pitch + slot_of(n)] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (NL) __syncthreads();                 // row_nl, G
+    bool big = false;
+    if (active) {
+        const double G = NL ? g_of_step : 0.0;
+        const float2 gl = NL ? g_lifted : f2(0.f, 0.f);
+#pragma unroll
+        for (int b = 0; b < kIncP; ++b) {
+            const int i = 1 + seg + b * lanes;
+            if (i < n) {
+                if constexpr (NL) {
+                    v[b] = calcnu_at<MODE, P3>(v[b], row_nl[P3 ? 0 : q], i, f3[P3 ? b : 0], gl, G);
+                    row[i] = v[b];
+                }
+                big = big || too_large(v[b].x) || too_large(v[b].y);
+                tile[at + slot_of(i)] = pack(lift(v[b]));
+            }
+        }
+    }
+    const int own = active ? seg : (threadIdx.x & 1);
+    if (__syncthreads_or(big)) {
+        double2 *t64 = reinterpret_cast<double2 *>(tile);
+        stage_coefs<MODE>(a, coef64);
+        if (active)
+            for (int i = 1 + seg; i < n; i += lanes) t64[at + slot_of(i)] = row[i];
+        __syncthreads();
+        const Share<kFp64, MODE> lane(a, coef64, own);
+        lane.template solve<kIncP, true>(
+            active, 1, [&](int i) { return t64[at + slot_of(i)]; }, 0, 0,
+            [&](int i, double2 u) { t64[at + slot_of(i)] = u; });
+        __syncthreads();
+        if (active)
+            for (int i = 1 + seg; i < n; i += lanes) row[i] = t64[at + slot_of(i)];
+        return;
+    }
+    const IncLane<MODE> lane(A, coef, own);
+    lane.template solve<true>(
+        active, 1, [&](int i) { return unpack(tile[at + slot_of(i)]); },
+        [&](int, int i, FC g) { tile[at + slot_of(i)] = pack(g); });
+    __syncthreads();
+    if (active) {
+#pragma unroll
+        for (int b = 0; b < kIncP; ++b) {
+            const int i = 1 + seg + b * lanes;
+            if (i < n) row[i] = plus<1, true>(row[i], unpack(tile[at + slot_of(i)]));
+        }
+    }
+}
+
+// y / z sweep: as k_split_yz; a lane reads the FP64 values of its rows again
+// (from L1 or L2) when it adds the increments.
+template <int MODE, bool NORM, bool NLOUT, bool P3, int THREADS>
+__global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_yz(const __grid_constant__ IncArgs A)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ double red[32], g_of_step;
+    __shared__ float2 g_lifted;
+    const SplitArgs<double> &a = A.s;
+    unsigned char *coef = smem_raw, *coef64 = coef + inc_coef_bytes(a.conv);
+    float4 *tile = reinterpret_cast<float4 *>(coef64 + coef_bytes<double>(a.conv));
+    const int n = a.n, XL = a.per;
+    const int xl = threadIdx.x & (XL - 1), seg = threadIdx.x / XL;
+    const int la = blockIdx.x * XL + xl, lb = blockIdx.y;
+    const bool active = la < a.lines_a && seg < 2 * a.S;
+    const IncLane<MODE> lane(A, coef, seg < 2 * a.S ? seg : (seg & 1));
+    const long long base = active ? (long long)la * a.stride_a + (long long)lb * a.stride_b : 0;
+    double2 *line = a.psi + base;
+    stage_inc<MODE>(A, coef);
+    if (NLOUT && threadIdx.x == 0) {
+        g_of_step = a.sg.value();
+        g_lifted = lifted_g(g_of_step);
+    }
+    auto at_of = [&](int i) { return slot_of(i) * XL + xl; };
+    bool big = false;
+    if (active) {
+        double2 p[kIncP];
+#pragma unroll
+        for (int q = 0; q < kIncP; ++q)
+            if (lane.first + q <= lane.last) p[q] = line[(long long)lane.row(lane.first + q) * a.pstride];
+#pragma unroll
+        for (int q = 0; q < kIncP; ++q)
+            if (lane.first + q <= lane.last) {
+                big = big || too_large(p[q].x) || too_large(p[q].y);
+                tile[at_of(lane.row(lane.first + q))] = pack(lift(p[q]));
+            }
+        if (seg == 0) tile[at_of(0)] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (seg == 1) tile[at_of(n)] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    big = __syncthreads_or(big);
+    Calcnu<double, MODE> nl{};
+    const double G = NLOUT ? g_of_step : 0.0;
+    const float2 gl = NLOUT ? g_lifted : f2(0.f, 0.f);
+    if (NLOUT && !P3 && active) nl.setup(a.px, a.py, a.pz, nullptr, nullptr, nullptr, la, lb, 0.0, nullptr);
+    double acc = 0.0;
+    auto finish = [&](int i, double2 u) {
+        const long long at = (long long)i * a.pstride;
+        if constexpr (NLOUT) {
+            double2 f = make_double2(0.0, 0.0);
+            if constexpr (P3) f = a.p3[base + at];
+            u = calcnu_at<MODE, P3>(u, nl, i, f, gl, G);
+        }
+        line[at] = u;
+        if (NORM) acc = fma(u.x, u.x, fma(u.y, u.y, acc));
+    };
+    if (big) {
+        double2 *t64 = reinterpret_cast<double2 *>(tile);
+        stage_coefs<MODE>(a, coef64);
+        if (active) {
+#pragma unroll
+            for (int q = 0; q < kIncP; ++q)
+                if (lane.first + q <= lane.last) {
+                    const int i = lane.row(lane.first + q);
+                    t64[at_of(i)] = line[(long long)i * a.pstride];
+                }
+        }
+        __syncthreads();
+        const Share<kFp64, MODE> lane64(a, coef64, seg < 2 * a.S ? seg : (seg & 1));
+        lane64.template solve<kIncP, false>(
+            active, XL, [&](int i) { return t64[at_of(i)]; }, 0, 0, finish);
+    } else {
+        lane.template solve<false>(
+            active, XL, [&](int i) { return unpack(tile[at_of(i)]); },
+            [&](int, int i, FC g) { finish(i, plus<1, false>(line[(long long)i * a.pstride], g)); });
+    }
+    if (NORM) {
+        if (a.lw && active) acc *= a.lw[la];
+        block_partial(active ? acc : 0.0, red, &a.partials[(long long)blockIdx.y * gridDim.x + blockIdx.x]);
+    }
+}
+
+template <int MODE, bool NL, bool P3> cudaError_t go_x(const SplitPlan &p, const IncArgs &a, cudaStream_t st)
+{
+    auto kern = p.threads <= 256 ? k_inc_x<MODE, NL, P3, 256> : k_inc_x<MODE, NL, P3, kSplitThreads>;
+    cudaError_t e = allow_smem(kern, p.smem);
+    if (e != cudaSuccess) return e;
+    kern<<<p.grid_x, p.threads, p.smem, st>>>(a);
+    return cudaGetLastError();
+}
+
+template <int MODE, bool NORM, bool NLOUT, bool P3>
+cudaError_t go_yz(const SplitPlan &p, const IncArgs &a, cudaStream_t st)
+{
+    auto kern = p.threads <= 256 ? k_inc_yz<MODE, NORM, NLOUT, P3, 256> : k_inc_yz<MODE, NORM, NLOUT, P3, kSplitThreads>;
+    cudaError_t e = allow_smem(kern, p.smem);
+    if (e != cudaSuccess) return e;
+    kern<<<dim3(p.grid_x, p.grid_y), p.threads, p.smem, st>>>(a);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+bool inc_applies(const AxisTables &ax) { return ax.kre <= kIncKappaImag && ax.kim <= kIncKappaReal; }
+
+size_t inc_extra_smem(int conv) { return inc_coef_bytes(conv); }
+
+cudaError_t launch_sweep_inc(const SplitPlan &p, int mode, void *psi, const AxisTables &ax, const SweepGeom &g,
+                             const NonlinArgs *nl, bool nlout, const Partials *norm_out, cudaStream_t st)
+{
+    IncArgs a{};
+    a.s = split_args<kFp64>(p, mode, psi, ax, g, nl, norm_out);
+    a.rinf = ff_expand(a.s.rinf);
+    for (int q = 0; q < kIncEnds; ++q) {
+        const double2 f = a.s.mid[q];
+        a.kmid[q] = ff_expand(mode == 0 ? make_double2(a.s.k * f.x, 0.0) : make_double2(-a.s.k * f.y, a.s.k * f.x));
+    }
+    // rows nearer than this reach the lane's own damped by less than 2^-26
+    const double r = std::hypot(a.s.rinf.x, a.s.rinf.y);
+    a.near = 1;
+    for (double q = r; q >= 0x1p-26; q *= r) ++a.near;
+    const bool p3 = a.s.p3 != nullptr, norm = norm_out != nullptr;
+    if (p.x) {
+        if (nlout || norm || (p3 && mode == 0)) return cudaErrorInvalidValue;
+        if (!nl) return mode == 0 ? go_x<0, false, false>(p, a, st) : go_x<1, false, false>(p, a, st);
+        if (mode == 0) return go_x<0, true, false>(p, a, st);
+        return p3 ? go_x<1, true, true>(p, a, st) : go_x<1, true, false>(p, a, st);
+    }
+    if ((nl && !nlout) || (norm && (mode == 1 || nlout)) || (nlout && mode == 0)) return cudaErrorInvalidValue;
+    if (mode == 0) return norm ? go_yz<0, true, false, false>(p, a, st) : go_yz<0, false, false, false>(p, a, st);
+    if (!nlout) return go_yz<1, false, false, false>(p, a, st);
+    return p3 ? go_yz<1, false, true, true>(p, a, st) : go_yz<1, false, true, false>(p, a, st);
+}
+
+}  // namespace gp

@@ -218,7 +218,9 @@ int sweep_blocks(const SweepGeom &g);
 struct SplitPlan {
     int P = 0, S = 0, W = 0;
     bool x = false;              // lines contiguous in memory
-    bool increment = false;      // complex64: the TMA path's arithmetic, else the exact path's
+    // complex64: the TMA path's arithmetic (else the exact path's); FP64:
+    // float-float increments (sscn_inc.cu; else FP64)
+    bool increment = false;
     int per = 0, threads = 0;    // lines per block, threads per block
     unsigned grid_x = 0, grid_y = 0;
     size_t smem = 0;
@@ -228,6 +230,13 @@ bool split_plan(int prec, const AxisTables &ax, const SweepGeom &g, SplitPlan &p
                 bool increment = false);
 int split_blocks(const SplitPlan &plan);
 int split_most_blocks(const SweepGeom &g);
+// FP64 psi with float-float increments (sscn_inc.cu): whether kappa allows it,
+// its shared memory beyond the FP64 form's, and the launch.
+bool inc_applies(const AxisTables &ax);
+size_t inc_extra_smem(int conv);
+cudaError_t launch_sweep_inc(const SplitPlan &plan, int mode, void *psi, const AxisTables &ax,
+                             const SweepGeom &g, const NonlinArgs *nl, bool nl_at_output,
+                             const Partials *norm_out, cudaStream_t st);
 // nl: calcnu on every loaded point (x), or with nl_at_output on every result
 // (real time, y / z); norm_out (imaginary time, y / z): as launch_sweep_yz.
 cudaError_t launch_sweep_split(const SplitPlan &plan, int prec, int mode, void *psi,

@@ -1,4 +1,4 @@
-"""Sub-line sweeps (sscn_split.cu): grids whose lines are cut into pieces that
+"""Sub-line sweeps (sscn_split.cu, sscn_inc.cu): grids whose lines are cut into pieces that
 many lanes solve.  Shapes put every remainder of that cut on some axis (one
 row, one row more or less than full pieces, a single piece), uneven tiles of
 neighbouring lines, and lines longer than a block of 8 rows a lane holds.
@@ -113,3 +113,54 @@ def test_symmetric_splitting_and_modulated_g(mode, prec, table, shape):
         got = s.psi().astype(np.complex128)
     want = oracle.step_ext(oracle_params(shape, h, dt, w, g, mode), psi0.copy(), steps, 0, True, g1, omega)
     assert rel_l2(got, want) <= (1e-12 if prec == gp.GP_C128 else steps * 4 * 2.0 ** -23)
+
+
+def special_state(shape, seed):
+    """Values whose significands sit where the FP64 <-> float-float conversions
+    carry or borrow: powers of two and their neighbours, ties at the 24th bit,
+    all-ones significands, zeros."""
+    rng = np.random.default_rng(seed)
+    m = np.array([0.0, 1.0, 2.0 - 2.0 ** -52, 1.0 + 2.0 ** -24, 1.0 + 2.0 ** -24 + 2.0 ** -52, 1.0 + 2.0 ** -23,
+                  1.0 + 2.0 ** -52, 2.0 - 2.0 ** -24, 2.0 - 2.0 ** -25, 1.5 + 2.0 ** -24 - 2.0 ** -52])
+
+    def part():
+        v = rng.choice(m, shape[::-1]) * 2.0 ** rng.integers(-3, 3, shape[::-1])
+        return v * rng.choice([-1.0, 1.0], shape[::-1])
+
+    a = part() + 1j * part()
+    a[:, :, 0] = a[:, 0, :] = 0
+    if shape[2] > 1:
+        a[0] = 0
+    return a
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("mode", [gp.GP_IMAG, gp.GP_REAL])
+@pytest.mark.parametrize("shape", [(34, 18, 17), (66, 130, 1)])
+@pytest.mark.parametrize("scale", [1.0, 2.0 ** 100, 2.0 ** 92, 2.0 ** -60])
+def test_fp64_conversions_at_their_corners(mode, shape, scale):
+    """Sweeps of special values, also where a block leaves the float-float
+    range (2^93) for FP64 and at the lower end of its full precision."""
+    require_gpu()
+    dt, steps = 1e-3, 2
+    h = spacing(shape, 0.02, dt)
+    psi0 = special_state(shape, 3) * scale
+    got = run(shape, h, dt, (0.0, 0.0, 0.0), 0.0, mode, gp.GP_C128, steps, psi0)
+    want = psi0.copy()
+    oracle.step(oracle_params(shape, h, dt, (0.0, 0.0, 0.0), 0.0, mode), want, steps)
+    assert rel_l2(got, want) <= 1e-12
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("mode", [gp.GP_IMAG, gp.GP_REAL])
+@pytest.mark.parametrize("g", [4.0, 4000.0, -50.0])
+def test_fp64_nonlinear_factor_on_both_sides_of_its_series(mode, g):
+    """dt g |psi|^2 below 2^-8 everywhere, on both sides of it, negative g."""
+    require_gpu()
+    shape, dt, steps = (40, 33, 20), 1e-3, 3
+    h = spacing(shape, 0.0125, dt)
+    psi0 = rand_state(shape, 21)
+    got = run(shape, h, dt, W3, g, mode, gp.GP_C128, steps, psi0)
+    want = psi0.copy()
+    oracle.step(oracle_params(shape, h, dt, W3, g, mode), want, steps)
+    assert rel_l2(got, want) <= 1e-12
