@@ -793,6 +793,7 @@ gp::ObsArgs obs_args(const gp_ctx *c)
     a.vz = a.vy + c->grid.ny;
     a.x2f = c->obs_tab32;
     a.vxf = c->obs_tab32 + (c->grid.nx + c->grid.ny + c->grid.nz);
+    a.hwy2 = 0.5 * c->w[1] * c->w[1];
     a.scale = c->scale;
     return a;
 }
@@ -1550,7 +1551,9 @@ int gp_launches_per_step(gp_ctx *c, int *per_step, int *per_observables)
 {
     if (!c) return fail(c, GP_EINVAL, "gp_launches_per_step: null context");
     if (per_step) *per_step = kernels_per_step(c);
-    if (per_observables) *per_observables = 3;   // line pass + two finish passes
+    if (per_observables)                         // the pass and its finish
+        *per_observables = 1 + gp::obs_finish_launches(
+            c->axial ? c->grid.ny : gp::obs_walk(c->prec, c->grid.nx, c->grid.ny, c->grid.nz).rows());
     return GP_OK;
 }
 

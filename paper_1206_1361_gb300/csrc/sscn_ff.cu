@@ -666,13 +666,13 @@ __global__ void k_ff_to_c128(double2 *__restrict__ dst, const float4 *__restrict
 
 // --------------------------------------------------------------- observables
 //
-// A thread owns one x and walks a chunk of kObsLines consecutive y-lines of
-// one plane (blocks over x segments, line chunks and planes; coalesced
+// A thread owns one x and walks a chunk of `walk` consecutive y-lines of one
+// plane (blocks over x segments, line chunks and planes; coalesced
 // 16-byte loads of the pairs): each point is loaded once as the thread's own
 // value and carried to the next line as that line's y-neighbour; the
 // x-neighbour comes from the next lane (lane 31 loads it), the z-neighbour
 // from the next plane, which that plane's blocks, resident at the same time,
-// find in L2.  Per point: a = |psi|^2, a^2, y_j^2 a, V_y(j) a and the
+// find in L2.  Per point: a = |psi|^2, a^2, y_j^2 a and the
 // neighbour terms R = Re(psi_next conj(psi)) along x, y, z (zero beyond the
 // last stored point), each a float-float product summed per thread in
 // float-float (TwoSum + Fast2Sum after every addition); the factors constant
@@ -689,28 +689,25 @@ __device__ __forceinline__ float2 lane_sum(C z)
 
 __global__ void __launch_bounds__(256)
 k_observables_ff(const float4 *__restrict__ psi, ObsArgs a, const float2 *__restrict__ x2ff,
-                 const float2 *__restrict__ vxff, double *__restrict__ rows)
+                 const float2 *__restrict__ vxff, int walk, double *__restrict__ rows)
 {
-    __shared__ float2 yt[2][kObsLines];
+    __shared__ float2 y2[kObsLines];
     __shared__ double red[8][8];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const int nx = a.nx, ny = a.ny, nz = a.nz;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j0 = blockIdx.y * kObsLines, j1 = min(j0 + kObsLines, ny);
+    const int j0 = blockIdx.y * walk, j1 = min(j0 + walk, ny);
     const int k = blockIdx.z;
-    for (int t = threadIdx.x; t < kObsLines && j0 + t < ny; t += blockDim.x) {
-        yt[0][t] = split(a.y2[j0 + t]);
-        yt[1][t] = split(a.vy[j0 + t]);
-    }
+    for (int t = threadIdx.x; t < walk && j0 + t < ny; t += blockDim.x) y2[t] = split(a.y2[j0 + t]);
     __syncthreads();
     const bool in = i < nx, has_z = nz > 1 && k + 1 < nz;
     const long long plane = (long long)nx * ny;
     const float4 *pk = psi + k * plane;
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
     auto cv = [](float4 v) { return C{f2(v.x, v.y), f2(v.z, v.w)}; };
-    float2 acc[7];                          // S0, Sy, SVy, S4, Rx, Ry, Rz
+    float2 acc[6];                          // S0, Sy, S4, Rx, Ry, Rz
 #pragma unroll
-    for (int q = 0; q < 7; ++q) acc[q] = f2(0.f, 0.f);
+    for (int q = 0; q < 6; ++q) acc[q] = f2(0.f, 0.f);
     auto put = [&](int q, float2 t) { acc[q] = s_norm(s_add(acc[q], t)); };
     float4 v4 = in ? pk[(long long)j0 * nx + i] : zero;
 #pragma unroll 2
@@ -727,18 +724,19 @@ k_observables_ff(const float4 *__restrict__ psi, ObsArgs a, const float2 *__rest
         const C v = cv(v4);
         const float2 am = abs2(v);
         put(0, am);
-        put(1, s_mul(yt[0][j - j0], am));
-        put(2, s_mul(yt[1][j - j0], am));
-        put(3, s_mul(am, am));
-        put(4, lane_sum(lmul(cv(nb4), v.hi, v.lo)));
-        put(5, lane_sum(lmul(cv(vn4), v.hi, v.lo)));
-        if (nz > 1) put(6, lane_sum(lmul(cv(vz4), v.hi, v.lo)));
+        put(1, s_mul(y2[j - j0], am));
+        put(2, s_mul(am, am));
+        put(3, lane_sum(lmul(cv(nb4), v.hi, v.lo)));
+        put(4, lane_sum(lmul(cv(vn4), v.hi, v.lo)));
+        if (nz > 1) put(5, lane_sum(lmul(cv(vz4), v.hi, v.lo)));
         v4 = vn4;
     }
     // S0, Sx, Sy, SVx + SVy, S4, Rx, Ry, Rz
     const float2 x2 = in ? x2ff[i] : f2(0.f, 0.f), vx = in ? vxff[i] : f2(0.f, 0.f);
-    float2 t8[8] = {acc[0], s_mul(x2, acc[0]), acc[1], s_norm(s_add(s_mul(vx, acc[0]), acc[2])),
-                    acc[3], acc[4], acc[5], acc[6]};
+    // (V_y is proportional to y^2)
+    float2 t8[8] = {acc[0], s_mul(x2, acc[0]), acc[1],
+                    s_norm(s_add(s_mul(vx, acc[0]), s_mul(split(a.hwy2), acc[1]))),
+                    acc[2], acc[3], acc[4], acc[5]};
 #pragma unroll
     for (int q = 0; q < 8; ++q)
 #pragma unroll
@@ -932,14 +930,11 @@ cudaError_t launch_ff_from_c128_grid(void *dst, const void *src, int nx, int ny,
 cudaError_t launch_observables_ff(const void *psi, const ObsArgs &a, const float2 *x2ff,
                                   const float2 *vxff, double *scratch, double *sums, cudaStream_t st)
 {
-    dim3 grid;
-    int threads = 0;
-    obs_walk_geometry(a.nx, a.ny, a.nz, grid, threads);
-    k_observables_ff<<<grid, threads, 0, st>>>((const float4 *)psi, a, x2ff, vxff, scratch);
+    const ObsWalk w = obs_walk(kCFF, a.nx, a.ny, a.nz);
+    k_observables_ff<<<w.grid, w.threads, 0, st>>>((const float4 *)psi, a, x2ff, vxff, w.walk, scratch);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const long long nrows = (long long)grid.x * grid.y * grid.z;
-    return launch_rows_finish(scratch, nrows, scratch + nrows * kObsWidth, sums, st);
+    return launch_rows_finish(scratch, w.rows(), scratch + w.rows() * kObsWidth, sums, st);
 }
 
 cudaError_t launch_ff_to_c128(void *dst, const void *src, long long count, const double *scale,

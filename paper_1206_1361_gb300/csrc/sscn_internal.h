@@ -269,20 +269,29 @@ struct ObsArgs {
     int nx, ny, nz;
     const double *x2, *y2, *z2, *vx, *vy, *vz;
     const float *x2f, *vxf;    // FP32 roundings of x2, vx (complex64 form)
+    double hwy2;               // omega_y^2 / 2 (vy = hwy2 y2)
     const double *scale;   // pending scale (device)
 };
 // Doubles of scratch launch_observables needs for this grid.
 long long obs_scratch_doubles(const ObsArgs &a);
-// Observables passes that walk y-lines (complex64, float-float): threads
-// along x (a multiple of 32, at most 256), blocks over (x segments, chunks of
-// kObsLines lines, planes); one row of sums per block.
+// Launch shape of an observables pass: threads along x (a multiple of 32, at
+// most 256), each walking `walk` (<= kObsLines) consecutive y-lines of a plane;
+// blocks over (x segments, line chunks, planes); one row of sums per block.
 constexpr int kObsLines = 64;
-void obs_walk_geometry(int nx, int ny, int nz, dim3 &grid, int &threads);
+struct ObsWalk {
+    dim3 grid;
+    int threads = 0, walk = 0;
+    long long rows() const { return (long long)grid.x * grid.y * grid.z; }
+};
+ObsWalk obs_walk(int prec, int nx, int ny, int nz);
 cudaError_t launch_observables(int prec, const void *psi, const ObsArgs &a,
                                double *scratch, double *sums, cudaStream_t st);
-// Fixed-order finish of `lines` partials rows of kObsWidth doubles into sums
-// (two passes through `stage`, ceil(lines / 1024) rows).
-cudaError_t launch_rows_finish(const double *rows, long long lines, double *stage, double *sums,
+// Fixed-order finish of `rows` partials rows of kObsWidth doubles into sums: one
+// launch, or two (through `stage`, obs_stage_rows rows) beyond kObsOneStage rows.
+constexpr int kObsOneStage = 1024;
+int obs_finish_launches(long long rows);
+long long obs_stage_rows(long long rows);
+cudaError_t launch_rows_finish(const double *rows, long long count, double *stage, double *sums,
                                cudaStream_t st);
 
 // ---- axially symmetric psi(rho, z) (sscn_axial.cu), FP64 ---------------------

@@ -421,34 +421,27 @@ __global__ void k_add_step(long long *step) { *step += 1; }
 
 // ------------------------------------------------------------ observables
 //
-// Per x-line (j, k), FP64 grids: one thread walks the line in order
-// (consecutive threads on consecutive lines; the line's points come through
-// L1).  Per point: a = |psi|^2, its x^2 and V_x weighted sums, |psi|^4, and the
-// neighbour terms along x, y and z (zero beyond the last stored point); the
-// y and z coordinate factors are constant on the line, so sum y^2 |psi|^2 =
-// y_j^2 sum |psi|^2 etc. are formed once per line.  Each line writes its 9
-// sums (times the pending scale s^2, s^4 for |psi|^4) to its own partials
-// row; two fixed-order passes add the rows, so the result does not depend on
-// the launch shape.  A thread per line keeps every sum in one thread: no
-// warp reduction per line, which on GB300 (2 FP64 FMA per clock per SM) cost
-// more than the points themselves.
+// Sums over the grid: |psi|^2, its x^2, y^2, z^2 and V weighted sums, |psi|^4,
+// and the neighbour terms along x, y and z (zero beyond the last stored
+// point), times the pending scale s^2 (s^4 for |psi|^4).
 //
-// FP64: the neighbour terms are R_k = sum Re(psi_next conj(psi)) (2 FMA),
-// and the finish forms K_k = 2 S0 - 2 R_k (every point is once "next" and
-// once "current", the boundary values are zero): sum |psi_next - psi|^2
-// exactly, with a relative rounding of ~1e-14 after the cancellation.
+// FP64: the neighbour terms are R_k = sum Re(psi_next conj(psi)) (2 FMA), and
+// the finish forms K_k = 2 S0 - 2 R_k (every point is once "next" and once
+// "current", the boundary values are zero): sum |psi_next - psi|^2 exactly,
+// with a relative rounding of ~1e-14 after the cancellation.  complex64 (FP32
+// terms) sums the differences (the cancellation would amplify FP32 rounding
+// past the 1e-6 the form is held to) with compensated partials per thread.
 //
-// complex64 (FP32 terms, memory-bound) keeps a warp per line for coalesced
-// loads and the differences (the cancellation would amplify FP32 rounding past
-// the 1e-6 the form is held to); its lanes' compensated FP32 partials are
-// combined across the warp in FP32 with an error-free sum (TwoSum), not in
-// FP64, and lane 0 converts the line's totals.
+// The passes are bound by the FP64 pipe (10 instructions a point at FP64) and,
+// on small grids, by the chain of a thread's walk and of the finish: the walk
+// shortens until there are blocks for every SM, and the finish gives each of
+// the 9 sums a warp of its own.  500 x 384 FP64: 419 us with a thread per whole
+// line and 9 sums one after the other in the finish.
 
 constexpr int kObsThreads = 256;
-constexpr int kObsChunk = 1024;          // lines per first-stage finish block
 
-// A thread owns one x and walks a chunk of kObsLines consecutive y-lines of
-// one plane (blocks over x segments, line chunks and planes): each point is
+// A thread owns one x and walks a chunk of `walk` consecutive y-lines of one
+// plane (blocks over x segments, line chunks and planes): each point is
 // loaded once as the thread's own value and carried to the next line as that
 // line's y-neighbour; the x-neighbour comes from the next lane (lane 31 loads
 // it), the z-neighbour from the next plane, which the blocks of that plane
@@ -531,75 +524,92 @@ k_observables_c64(const float2 *__restrict__ psi, ObsArgs a, double *__restrict_
     }
 }
 
-// Thread per line (FP64 grids).
-template <typename T>
+// FP64 grids, the same walk.  Per point 11 FP64 instructions: V_y is
+// proportional to y^2, so its sum is the y^2 sum times omega_y^2 / 2.  The
+// threads' sums meet in shared memory, a warp per quantity (a shuffle tree per
+// warp and quantity would cost more FP64-pipe time than a short walk).
 __global__ void __launch_bounds__(kObsThreads)
-k_observables(const typename CT<T>::c *__restrict__ psi, ObsArgs a,
-              double *__restrict__ partials)
+k_observables_f64(const double2 *__restrict__ psi, ObsArgs a, int walk, double *__restrict__ rows)
 {
-    using C = typename CT<T>::c;
-    const long long line = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    constexpr int kQ = 7;                    // S0, Sx, Sy, S4, Rx, Ry, Rz
+    __shared__ double y2[kObsLines], part[kQ][kObsThreads], red[kQ];
+    const int lane = threadIdx.x & 31;
     const int nx = a.nx, ny = a.ny, nz = a.nz;
-    if (line >= (long long)ny * nz) return;
-    const int j = (int)(line % ny), k = (int)(line / ny);
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int j0 = blockIdx.y * walk, j1 = min(j0 + walk, ny);
+    const int k = blockIdx.z;
+    for (int t = threadIdx.x; t < walk && j0 + t < ny; t += blockDim.x) y2[t] = a.y2[j0 + t];
+    __syncthreads();
+    const bool in = i < nx, has_z = k + 1 < nz;
     const long long plane = (long long)nx * ny;
-    const C *row = psi + line * nx;
-    const bool has_y = j + 1 < ny, has_z = nz > 1 && k + 1 < nz;
-    const T *x2 = sizeof(T) == 8 ? (const T *)a.x2 : (const T *)a.x2f;
-    const T *vx = sizeof(T) == 8 ? (const T *)a.vx : (const T *)a.vxf;
-    constexpr bool RFORM = sizeof(T) == 8;
-    Acc<T> s0, sx, svx, s4, kx, ky, kz;
-    const C zero = mk<T>((T)0, (T)0);
-    C v = row[0];
-    for (int i = 0; i < nx; ++i) {
-        const C nb = (i + 1 < nx) ? row[i + 1] : zero;
-        const C ny_ = has_y ? row[i + nx] : zero;
-        const C nz_ = has_z ? row[i + plane] : zero;
-        const T am = fma(v.x, v.x, v.y * v.y);
-        s0.add(am);
-        sx.add_prod(x2[i], am);
-        svx.add_prod(vx[i], am);
-        s4.add_prod(am, am);
-        if constexpr (RFORM) {
-            kx.s = fma(nb.x, v.x, fma(nb.y, v.y, kx.s));
-            ky.s = fma(ny_.x, v.x, fma(ny_.y, v.y, ky.s));
-            kz.s = fma(nz_.x, v.x, fma(nz_.y, v.y, kz.s));
-        } else {
-            kx.add_sq2(nb.x - v.x, nb.y - v.y);
-            ky.add_sq2(ny_.x - v.x, ny_.y - v.y);
-            if (nz > 1) kz.add_sq2(nz_.x - v.x, nz_.y - v.y);
-        }
-        v = nb;
+    const double2 *pk = psi + k * plane;
+    const double2 zero = make_double2(0.0, 0.0);
+    double s0 = 0.0, sy = 0.0, s4 = 0.0, rx = 0.0, ry = 0.0, rz = 0.0;
+    double2 v = in ? pk[(long long)j0 * nx + i] : zero;
+#pragma unroll 4
+    for (int j = j0; j < j1; ++j) {
+        const long long at = (long long)j * nx + i;
+        const double2 vn = (in && j + 1 < ny) ? pk[at + nx] : zero;     // y-neighbour
+        const double2 vz = (in && has_z) ? pk[at + plane] : zero;        // z-neighbour
+        double2 nb;                                                      // x-neighbour
+        nb.x = __shfl_down_sync(0xffffffffu, v.x, 1);
+        nb.y = __shfl_down_sync(0xffffffffu, v.y, 1);
+        if (lane == 31) nb = (i + 1 < nx) ? pk[at + 1] : zero;
+        const double am = fma(v.x, v.x, v.y * v.y);
+        s0 += am;
+        sy = fma(y2[j - j0], am, sy);
+        s4 = fma(am, am, s4);
+        rx = fma(nb.x, v.x, fma(nb.y, v.y, rx));
+        ry = fma(vn.x, v.x, fma(vn.y, v.y, ry));
+        rz = fma(vz.x, v.x, fma(vz.y, v.y, rz));
+        v = vn;
     }
-    const double sc = *a.scale, s2 = sc * sc;
-    const double r0 = s0.get();
-    double *out = partials + line * kObsWidth;
-    out[0] = s2 * r0;
-    out[1] = s2 * sx.get();
-    out[2] = s2 * a.y2[j] * r0;
-    out[3] = s2 * a.z2[k] * r0;
-    out[4] = s2 * (svx.get() + (a.vy[j] + a.vz[k]) * r0);
-    out[5] = s2 * s2 * s4.get();
-    out[6] = s2 * kx.get();
-    out[7] = s2 * ky.get();
-    out[8] = s2 * kz.get();
+    const double q[kQ] = {s0, in ? a.x2[i] * s0 : 0.0, sy, s4, rx, ry, rz};
+#pragma unroll
+    for (int t = 0; t < kQ; ++t) part[t][threadIdx.x] = q[t];
+    __syncthreads();
+    for (int t = threadIdx.x >> 5; t < kQ; t += blockDim.x >> 5) {
+        double r = 0.0;
+        for (int w = lane; w < blockDim.x; w += 32) r += part[t][w];
+        r = warp_sum(r);
+        if (lane == 0) red[t] = r;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const double sc = *a.scale, s2 = sc * sc;
+        // V_x likewise: omega_x^2 / 2 times the x^2 sum (the table's ratio at the
+        // first point, which is not the origin)
+        const double hwx2 = a.vx[0] / a.x2[0];
+        double *out = rows + (((long long)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * kObsWidth;
+        out[0] = s2 * red[0];
+        out[1] = s2 * red[1];
+        out[2] = s2 * red[2];
+        out[3] = s2 * a.z2[k] * red[0];
+        out[4] = s2 * (fma(hwx2, red[1], a.hwy2 * red[2]) + a.vz[k] * red[0]);
+        out[5] = s2 * s2 * red[3];
+        out[6] = s2 * red[4];
+        out[7] = s2 * red[5];
+        out[8] = s2 * red[6];
+    }
 }
 
-// Sum rows [b * chunk, (b + 1) * chunk) of a [rows][9] array into out[b][9].
-__global__ void __launch_bounds__(256)
+// Sum rows [b chunk, (b + 1) chunk) of a [count][9] array into out[b][9], a warp
+// per column, four interleaved chains a lane.
+__global__ void __launch_bounds__(32 * kObsWidth)
 k_rows_sum(const double *__restrict__ rows, long long count, int chunk,
            double *__restrict__ out)
 {
-    __shared__ double red[32];
+    const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
     const long long r0 = (long long)blockIdx.x * chunk;
-    long long r1 = r0 + chunk;
-    if (r1 > count) r1 = count;
-    for (int q = 0; q < kObsWidth; ++q) {
-        double v = 0.0;
-        for (long long r = r0 + threadIdx.x; r < r1; r += blockDim.x) v += rows[r * kObsWidth + q];
-        const double t = block_sum(v, red);
-        if (threadIdx.x == 0) out[(long long)blockIdx.x * kObsWidth + q] = t;
-    }
+    const long long r1 = r0 + chunk < count ? r0 + chunk : count;
+    double v[4] = {0.0, 0.0, 0.0, 0.0};
+    long long r = r0 + lane;
+    for (; r + 96 < r1; r += 128)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] += rows[(r + 32 * u) * kObsWidth + q];
+    for (; r < r1; r += 32) v[0] += rows[r * kObsWidth + q];
+    const double t = warp_sum((v[0] + v[1]) + (v[2] + v[3]));
+    if (lane == 0) out[(long long)blockIdx.x * kObsWidth + q] = t;
 }
 
 constexpr int kPointThreads = 256;
@@ -755,57 +765,68 @@ cudaError_t launch_add_step(long long *step, cudaStream_t st)
     return cudaGetLastError();
 }
 
-void obs_walk_geometry(int nx, int ny, int nz, dim3 &grid, int &threads)
+ObsWalk obs_walk(int prec, int nx, int ny, int nz)
 {
-    threads = 32 * ((nx + 31) / 32);
-    if (threads > 256) threads = 256;
-    grid = dim3((unsigned)((nx + threads - 1) / threads), (unsigned)((ny + kObsLines - 1) / kObsLines),
-                (unsigned)nz);
+    ObsWalk w;
+    w.threads = 32 * ((nx + 31) / 32);
+    if (w.threads > kObsThreads) w.threads = kObsThreads;
+    // 64 lines (measured best of 8 .. 256 on large grids), fewer while there
+    // would be fewer blocks than SMs; complex64 always 64: its FP32 partials per
+    // thread round at 2^-24, so another walk would show in the FP64 results
+    // (7e-10 on 756 x 526)
+    for (w.walk = kObsLines;; w.walk /= 2) {
+        w.grid = dim3((unsigned)((nx + w.threads - 1) / w.threads), (unsigned)((ny + w.walk - 1) / w.walk), (unsigned)nz);
+        if (prec == kC64 || w.walk == 4 || w.rows() >= 152) return w;
+    }
+}
+
+int obs_finish_launches(long long rows) { return rows > kObsOneStage ? 2 : 1; }
+
+namespace {
+int obs_chunk(long long rows)
+{
+    const long long c = (rows + kObsOneStage - 1) / kObsOneStage;
+    return (int)(c > 128 ? c : 128);
+}
+}
+
+long long obs_stage_rows(long long rows)
+{
+    return rows > kObsOneStage ? (rows + obs_chunk(rows) - 1) / obs_chunk(rows) : 0;
 }
 
 long long obs_scratch_doubles(const ObsArgs &a)
 {
-    dim3 grid;
-    int threads = 0;
-    obs_walk_geometry(a.nx, a.ny, a.nz, grid, threads);
-    long long rows = (long long)a.ny * a.nz;       // a row per line (FP64)
-    const long long walk = (long long)grid.x * grid.y * grid.z;
-    if (walk > rows) rows = walk;
-    const long long chunks = (rows + kObsChunk - 1) / kObsChunk;
-    return (rows + chunks) * kObsWidth;
+    long long rows = obs_walk(kC128, a.nx, a.ny, a.nz).rows();      // the most of any precision
+    if (a.nz == 1 && a.ny > rows) rows = a.ny;      // the axial form: a row per line
+    return (rows + obs_stage_rows(rows)) * kObsWidth;
 }
 
 cudaError_t launch_observables(int prec, const void *psi, const ObsArgs &a,
                                double *scratch, double *sums, cudaStream_t st)
 {
-    const long long lines = (long long)a.ny * a.nz;
-    double *rows = scratch, *stage = scratch + lines * kObsWidth;
-    if (prec == kC128) {
-        const long long blocks = (lines + kObsThreads - 1) / kObsThreads;
-        k_observables<double><<<(unsigned)blocks, kObsThreads, 0, st>>>((const double2 *)psi, a, rows);
-    } else {
-        dim3 grid;
-        int threads = 0;
-        obs_walk_geometry(a.nx, a.ny, a.nz, grid, threads);
-        k_observables_c64<<<grid, threads, 0, st>>>((const float2 *)psi, a, rows);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        const long long nrows = (long long)grid.x * grid.y * grid.z;
-        return launch_rows_finish(rows, nrows, rows + nrows * kObsWidth, sums, st);
-    }
+    const ObsWalk w = obs_walk(prec, a.nx, a.ny, a.nz);
+    if (prec == kC128)
+        k_observables_f64<<<w.grid, w.threads, 0, st>>>((const double2 *)psi, a, w.walk, scratch);
+    else
+        k_observables_c64<<<w.grid, w.threads, 0, st>>>((const float2 *)psi, a, scratch);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    return launch_rows_finish(rows, lines, stage, sums, st);
+    return launch_rows_finish(scratch, w.rows(), scratch + w.rows() * kObsWidth, sums, st);
 }
 
-cudaError_t launch_rows_finish(const double *rows, long long lines, double *stage, double *sums,
+cudaError_t launch_rows_finish(const double *rows, long long count, double *stage, double *sums,
                                cudaStream_t st)
 {
-    const long long chunks = (lines + kObsChunk - 1) / kObsChunk;
-    k_rows_sum<<<(unsigned)chunks, 256, 0, st>>>(rows, lines, kObsChunk, stage);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_rows_sum<<<1, 256, 0, st>>>(stage, chunks, (int)chunks, sums);
+    if (count > kObsOneStage) {
+        const long long chunks = obs_stage_rows(count);
+        k_rows_sum<<<(unsigned)chunks, 32 * kObsWidth, 0, st>>>(rows, count, obs_chunk(count), stage);
+        cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        rows = stage;
+        count = chunks;
+    }
+    k_rows_sum<<<1, 32 * kObsWidth, 0, st>>>(rows, count, (int)count, sums);
     return cudaGetLastError();
 }
 

@@ -164,3 +164,20 @@ def test_fp64_nonlinear_factor_on_both_sides_of_its_series(mode, g):
     want = psi0.copy()
     oracle.step(oracle_params(shape, h, dt, W3, g, mode), want, steps)
     assert rel_l2(got, want) <= 1e-12
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("shape", [(3, 3, 3), (33, 5, 4), (257, 3, 1), (64, 65, 9), (500, 129, 1), (40, 70, 300)])
+@pytest.mark.parametrize("prec", [gp.GP_C128, gp.GP_CFF])
+def test_fp64_observables_of_every_walk(shape, prec):
+    """Walks of 4 to 64 lines, ragged x segments and line chunks, one and two
+    finish launches: N, mu, E and the rms sizes of a random state against the
+    oracle within 1e-12 (FP64: a few hundred roundings; pairs: 2^-46 a term)."""
+    require_gpu()
+    h, dt, g, w = (0.2, 0.25, 0.3), 1e-3, 5.0, trap_of(shape)
+    psi0 = rand_state(shape, 13)
+    with gp.Solver(shape, h, dt, *w, g, gp.GP_REAL, prec) as s:
+        got = s.load(psi0).observables()
+    want = oracle.observables(oracle_params(shape, h, dt, w, g, gp.GP_REAL), psi0)
+    for k in ("norm", "mu", "energy", "rms_x", "rms_y", "rms_z", "rms_r"):
+        assert abs(got[k] - want[k]) <= 1e-12 * abs(want[k]), k
