@@ -431,8 +431,8 @@ void gp_destroy(gp_ctx *ctx);
  * A batch advances many independent problems -- each with its own grid
  * (edges 3 .. 512 for complex64, 3 .. 384 for complex128), spacings, trap
  * frequencies, g, dt and mode -- together: gp_batch_step runs n SSCN steps of
- * every instance in one persistent kernel launch (per 2^30 work items), whose
- * work items are (step, sweep or norm, instance, tile of 32 lines).  Each
+ * every instance, a launch per sweep (or one persistent kernel launch per 2^30
+ * work items, gp_batch_set_wait_ns) over tiles of 16 or 8 lines.  Each
  * instance follows the same discretisation as a context (calcnu, calclux,
  * calcluy, calcluz, calcnorm; observables calcmuen, calcrms), with the
  * elimination done exactly in shared memory, so its result does not depend
@@ -459,17 +459,19 @@ int gp_batch_set_params(gp_batch *b, int slot, double g, int mode);
 /* Advance every instance in the batch by n steps (asynchronous). */
 int gp_batch_step(gp_batch *b, int64_t n);
 /*
- * Budget, in nanoseconds of %globaltimer, of each dependency wait of the
- * batch's persistent kernel (a work item of one sweep waits until every item
- * of its instance's previous sweep has completed); default 2e9.  The paper
- * has no counterpart: this is failure detection for the persistent kernel.
- * A wait that exceeds its budget sets the batch's abort flag, every warp
- * leaves at its next item, and the next synchronising call (gp_batch_sync,
- * gp_batch_observables, gp_batch_store) returns GP_ETIMEOUT once; the steps
- * of that launch are then incomplete, so reload the instances before
- * stepping on.  ns = 0 makes every wait that is not satisfied at once give
- * up (used to test the path).  Takes effect at the next gp_batch_step.
- * GP_EINVAL for ns < 0.
+ * Run the batch's steps as one persistent launch per gp_batch_step from now on,
+ * with this budget, in nanoseconds of %globaltimer, for each dependency wait (a
+ * work item of one sweep waits until every item of its instance's previous
+ * sweep has completed).  Without this call a step is a launch per sweep, which
+ * the stream orders: faster, with no wait that could give up, and with the
+ * same results bit for bit.  The paper has no counterpart: this is failure
+ * detection for the persistent launch.  A wait that exceeds its budget sets the
+ * batch's abort flag, every warp leaves at its next item, and the next
+ * synchronising call (gp_batch_sync, gp_batch_observables, gp_batch_store)
+ * returns GP_ETIMEOUT once; the steps of that launch are then incomplete, so
+ * reload the instances before stepping on.  ns = 0 makes every wait that is
+ * not satisfied at once give up (used to test the path).  Takes effect at the
+ * next gp_batch_step.  GP_EINVAL for ns < 0.
  */
 int gp_batch_set_wait_ns(gp_batch *b, int64_t ns);
 /* Observables of every instance, out[slot] for slot < capacity (unused slots

@@ -181,3 +181,36 @@ def test_fp64_observables_of_every_walk(shape, prec):
     want = oracle.observables(oracle_params(shape, h, dt, w, g, gp.GP_REAL), psi0)
     for k in ("norm", "mu", "energy", "rms_x", "rms_y", "rms_z", "rms_r"):
         assert abs(got[k] - want[k]) <= 1e-12 * abs(want[k]), k
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("prec", [gp.GP_C64, gp.GP_C128])
+def test_batch_launch_forms_agree_bit_for_bit(prec):
+    """A launch per sweep and the persistent launch (selected by a wait
+    budget): the same tiles and arithmetic, the same bits; states stored to a
+    device buffer and to the host are the same."""
+    require_gpu()
+    import torch
+    dtype = torch.complex64 if prec == gp.GP_C64 else torch.complex128
+    shapes = [(33, 20, 17, 0), (96, 40, 1, 1), (130, 97, 12, 0), (48, 112, 33, 1)]
+    got = []
+    for queue in (False, True):
+        with gp.Batch(prec, cap_bytes=1 << 31) as b:
+            if queue:
+                b.set_wait_ns(2 * 10 ** 9)
+            slots = [b.add((nx, ny, nz), (0.2, 0.22, 0.25), 0.004, 1.0, 1.2, 1.5 if nz > 1 else 0.0, 8.0, mode,
+                           psi=rand_state((nx, ny, nz), 31).astype(np.complex64 if prec == gp.GP_C64 else np.complex128))
+                     for nx, ny, nz, mode in shapes]
+            b.step(5)
+            obs = b.observables()
+            out = []
+            for s, (nx, ny, nz, _) in zip(slots, shapes):
+                dev = torch.empty(nx * ny * nz, dtype=dtype, device="cuda")
+                gp.gp_batch_store(b.b, s, dev)
+                host = b.psi(s)
+                assert np.array_equal(dev.cpu().numpy().reshape(host.shape), host)
+                out.append(host)
+            got.append((out, obs))
+    for a, c in zip(got[0][0], got[1][0]):
+        assert np.array_equal(a, c)
+    assert got[0][1] == got[1][1]
