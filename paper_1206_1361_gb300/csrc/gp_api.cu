@@ -202,6 +202,7 @@ int upload_tables(gp_ctx *c)
             GP_CK(c, cudaMemcpy(d_mult64, mult.data(), m * sizeof(double2), cudaMemcpyHostToDevice));
             GP_CK(c, cudaMemcpy(d_cp32, cp32.data(), m * sizeof(float4), cudaMemcpyHostToDevice));
             GP_CK(c, cudaMemcpy(d_mult32, mult32.data(), m * sizeof(float4), cudaMemcpyHostToDevice));
+            a.settled = true;          // (the copies are synchronous)
             if (is_ff(c)) {
                 gp::FfAxis &f = c->ffax[mode][k];
                 gp::FfCoef *d_cp = f.cp, *d_mult = f.mult;

@@ -43,6 +43,7 @@
 #include "sscn_internal.h"
 #include "sscn_line.cuh"
 #include "sscn_pair.cuh"
+#include "sscn_pdl.cuh"
 #include "sscn_seg.cuh"
 
 namespace {
@@ -459,6 +460,8 @@ __global__ void __launch_bounds__(32) k_batch_tiles(const __grid_constant__ Laun
     const int *pr = A.pref + P * (A.N + 1);
     const int i = find_instance(pr, A.N, (int)blockIdx.x, threadIdx.x), tile = (int)blockIdx.x - pr[i];
     const Inst &I = A.inst[i];
+    // (the launch structures are in place before a step's first kernel starts)
+    gp::pdl_wait();
     if (I.rows[P] == kSegLines) sweep_tile<T, kSegLines>(I, P, tile, sm, threadIdx.x);
     else sweep_tile<T, kPairLines>(I, P, tile, sm, threadIdx.x);
 }
@@ -467,6 +470,7 @@ __global__ void __launch_bounds__(32) k_batch_tiles(const __grid_constant__ Laun
 __global__ void __launch_bounds__(32) k_batch_norm(const __grid_constant__ LaunchArgs A)
 {
     const Inst &I = A.inst[blockIdx.x];
+    gp::pdl_wait();
     if (I.mode == 0) norm_item(I, threadIdx.x, A.err);
 }
 
@@ -1054,8 +1058,7 @@ template <typename T, int P> cudaError_t launch_tiles(gp_batch *b)
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->smem);
     if (e != cudaSuccess) return e;
-    kern<<<(unsigned)b->args.phase_total[P], 32, b->smem, b->stream>>>(b->args);
-    return cudaGetLastError();
+    return gp::launch_after(true, kern, (unsigned)b->args.phase_total[P], 32, b->smem, b->stream, b->args);
 }
 
 void stepped(gp_batch *b, int64_t n)
@@ -1073,8 +1076,7 @@ template <typename T> int enqueue_step(gp_batch *b)
     GP_BCK(b, (launch_tiles<T, 1>(b)));
     GP_BCK(b, (launch_tiles<T, 2>(b)));
     if (b->args.phase_total[3]) {
-        k_batch_norm<<<b->args.N, 32, 0, b->stream>>>(b->args);
-        GP_BCK(b, cudaGetLastError());
+        GP_BCK(b, gp::launch_after(true, k_batch_norm, (unsigned)b->args.N, 32, 0, b->stream, b->args));
     }
     return GP_OK;
 }

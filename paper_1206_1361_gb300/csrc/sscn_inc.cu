@@ -342,6 +342,11 @@ __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_x(const __
     const bool active = q < rows;
     const int at = (active ? q : 0) * pitch;
     double2 *row = a.psi + (long long)(line0 + (active ? q : 0)) * n;
+    // (tables and set-up before the wait for the kernel before this one)
+    stage_inc<MODE>(A, coef);
+    for (int r = threadIdx.x; r < a.per; r += blockDim.x)
+        tile[r * pitch] = tile[r * pitch + slot_of(n)] = make_float4(0.f, 0.f, 0.f, 0.f);
+    pdl_wait();
     double2 v[kIncP], f3[NL && P3 ? kIncP : 1];
     if (active) {
 #pragma unroll
@@ -363,9 +368,6 @@ __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_x(const __
             const int L = line0 + r;
             row_nl[r].setup(a.px, a.py, a.pz, nullptr, nullptr, nullptr, L % a.lines_a, L / a.lines_a, 0.0, a.scale);
         }
-    stage_inc<MODE>(A, coef);
-    for (int r = threadIdx.x; r < a.per; r += blockDim.x)
-        tile[r * pitch] = tile[r * pitch + slot_of(n)] = make_float4(0.f, 0.f, 0.f, 0.f);
     if (NL) __syncthreads();                 // row_nl, G
     bool big = false;
     if (active) {
@@ -433,6 +435,7 @@ __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_yz(const _
     const long long base = active ? (long long)la * a.stride_a + (long long)lb * a.stride_b : 0;
     double2 *line = a.psi + base;
     stage_inc<MODE>(A, coef);
+    pdl_wait();
     if (NLOUT && threadIdx.x == 0) {
         g_of_step = a.sg.value();
         g_lifted = lifted_g(g_of_step);
@@ -500,8 +503,7 @@ template <int MODE, bool NL, bool P3> cudaError_t go_x(const SplitPlan &p, const
     auto kern = p.threads <= 256 ? k_inc_x<MODE, NL, P3, 256> : k_inc_x<MODE, NL, P3, kSplitThreads>;
     cudaError_t e = allow_smem(kern, p.smem);
     if (e != cudaSuccess) return e;
-    kern<<<p.grid_x, p.threads, p.smem, st>>>(a);
-    return cudaGetLastError();
+    return launch_after(p.after, kern, p.grid_x, p.threads, p.smem, st, a);
 }
 
 template <int MODE, bool NORM, bool NLOUT, bool P3>
@@ -510,8 +512,7 @@ cudaError_t go_yz(const SplitPlan &p, const IncArgs &a, cudaStream_t st)
     auto kern = p.threads <= 256 ? k_inc_yz<MODE, NORM, NLOUT, P3, 256> : k_inc_yz<MODE, NORM, NLOUT, P3, kSplitThreads>;
     cudaError_t e = allow_smem(kern, p.smem);
     if (e != cudaSuccess) return e;
-    kern<<<dim3(p.grid_x, p.grid_y), p.threads, p.smem, st>>>(a);
-    return cudaGetLastError();
+    return launch_after(p.after, kern, dim3(p.grid_x, p.grid_y), p.threads, p.smem, st, a);
 }
 
 }  // namespace

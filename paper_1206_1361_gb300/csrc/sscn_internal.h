@@ -34,6 +34,9 @@ struct AxisTables {
     // Look-back window of the TMA path: smallest W with max|c'|^(W+1) below
     // 2^-55 (FP64) / 2^-40 (complex64); 0 if none up to 64.
     int win64 = 0, win32 = 0;
+    // The device tables were complete before anything now in the stream: a
+    // kernel may read them before the kernel ahead of it has ended.
+    bool settled = false;
 };
 
 // Compute both table sets of one axis on the host and every derived field
@@ -218,6 +221,7 @@ int sweep_blocks(const SweepGeom &g);
 struct SplitPlan {
     int P = 0, S = 0, W = 0;
     bool x = false;              // lines contiguous in memory
+    bool after = false;          // programmatic dependent launch (the axis' tables are settled)
     // complex64: the TMA path's arithmetic (else the exact path's); FP64:
     // float-float increments (sscn_inc.cu; else FP64)
     bool increment = false;

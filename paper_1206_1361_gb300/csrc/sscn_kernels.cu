@@ -21,6 +21,7 @@
 #include "sscn_accum.cuh"
 #include "sscn_internal.h"
 #include "sscn_line.cuh"
+#include "sscn_pdl.cuh"
 
 namespace gp {
 namespace {
@@ -287,6 +288,7 @@ __global__ void k_norm_finish(const double *__restrict__ partials, int count,
 {
     __shared__ double red[32];
     double v = 0.0;
+    pdl_wait();
     for (int i = threadIdx.x; i < count; i += blockDim.x) v += partials[i];
     const double total = block_sum(v, red);
     if (threadIdx.x == 0) {
@@ -417,7 +419,11 @@ __global__ void k_build_pot3(double2 *__restrict__ p3, const double2 *__restrict
 }
 
 __global__ void k_set_step(long long *step, long long value) { *step = value; }
-__global__ void k_add_step(long long *step) { *step += 1; }
+__global__ void k_add_step(long long *step)
+{
+    pdl_wait();
+    *step += 1;
+}
 
 // ------------------------------------------------------------ observables
 //
@@ -679,8 +685,7 @@ cudaError_t launch_sweep_yz(int prec, int mode, void *psi, void *work,
 cudaError_t launch_norm_finish(const double *partials, int count, double w,
                                double *scale, double *norm_out, int *err, cudaStream_t st)
 {
-    k_norm_finish<<<1, 256, 0, st>>>(partials, count, w, scale, norm_out, err);
-    return cudaGetLastError();
+    return launch_after(true, k_norm_finish, 1, 256, 0, st, partials, count, w, scale, norm_out, err);
 }
 
 cudaError_t launch_apply_scale(int prec, void *psi, long long count, double *scale,
@@ -761,8 +766,7 @@ cudaError_t launch_set_step(long long *step, long long value, cudaStream_t st)
 
 cudaError_t launch_add_step(long long *step, cudaStream_t st)
 {
-    k_add_step<<<1, 1, 0, st>>>(step);
-    return cudaGetLastError();
+    return launch_after(true, k_add_step, 1, 1, 0, st, step);
 }
 
 ObsWalk obs_walk(int prec, int nx, int ny, int nz)

@@ -205,6 +205,8 @@ __global__ void __launch_bounds__(kSplitThreads) k_split_x(const __grid_constant
     const int line0 = blockIdx.x * a.per;
     const int rows = min(a.per, a.lines_a * a.lines_b - line0);
     __shared__ double g_of_step;
+    stage_coefs<MODE>(a, smem_raw);
+    pdl_wait();
     if (P3 && threadIdx.x == 0) g_of_step = a.sg.value();
     if (NL && !P3)
         for (int q = threadIdx.x; q < rows; q += blockDim.x) {
@@ -212,7 +214,6 @@ __global__ void __launch_bounds__(kSplitThreads) k_split_x(const __grid_constant
             row_nl[q].setup(a.px, a.py, a.pz, a.tx, a.ty, a.tz, L % a.lines_a, L / a.lines_a, a.sg.value(),
                             a.scale);
         }
-    stage_coefs<MODE>(a, smem_raw);
     if (FORM == kIncrement)
         for (int q = threadIdx.x; q < a.per; q += blockDim.x)
             tile[q * pitch] = tile[q * pitch + slot_of(n)] = cx<T>((T)0, (T)0);
@@ -293,6 +294,8 @@ __global__ void __launch_bounds__(kSplitThreads) k_split_yz(const __grid_constan
     __shared__ double red[32], g_of_step;
     using Lane = Share<FORM, MODE>;
     C *tile = reinterpret_cast<C *>(smem_raw + coef_bytes<T>(a.conv)), *dtile = tile + a.per * (slot_of(a.n) + 1);
+    stage_coefs<MODE>(a, smem_raw);
+    pdl_wait();
     if (NLOUT && threadIdx.x == 0) g_of_step = a.sg.value();
     const int n = a.n, XL = a.per;
     const int xl = threadIdx.x & (XL - 1), seg = threadIdx.x / XL;
@@ -309,7 +312,6 @@ __global__ void __launch_bounds__(kSplitThreads) k_split_yz(const __grid_constan
         for (int q = 0; q < kOwn; ++q)
             if (lane.first + q <= lane.last) p[q] = line[(long long)lane.row(lane.first + q) * a.pstride];
     }
-    stage_coefs<MODE>(a, smem_raw);
     if (active) {
 #pragma unroll
         for (int q = 0; q < kOwn; ++q)
@@ -353,8 +355,7 @@ cudaError_t go_x(const SplitPlan &p, const SplitArgs<T> &a, cudaStream_t st)
     auto kern = k_split_x<FORM, MODE, NL, P3, P>;
     cudaError_t e = allow_smem(kern, p.smem);
     if (e != cudaSuccess) return e;
-    kern<<<p.grid_x, p.threads, p.smem, st>>>(a);
-    return cudaGetLastError();
+    return launch_after(p.after, kern, p.grid_x, p.threads, p.smem, st, a);
 }
 
 template <int FORM, int MODE, bool NORM, bool NLOUT, bool P3, int P, typename T>
@@ -363,8 +364,7 @@ cudaError_t go_yz(const SplitPlan &p, const SplitArgs<T> &a, cudaStream_t st)
     auto kern = k_split_yz<FORM, MODE, NORM, NLOUT, P3, P>;
     cudaError_t e = allow_smem(kern, p.smem);
     if (e != cudaSuccess) return e;
-    kern<<<dim3(p.grid_x, p.grid_y), p.threads, p.smem, st>>>(a);
-    return cudaGetLastError();
+    return launch_after(p.after, kern, dim3(p.grid_x, p.grid_y), p.threads, p.smem, st, a);
 }
 
 template <int FORM, int MODE, int P, typename T>
@@ -478,6 +478,7 @@ bool split_plan(int prec, const AxisTables &ax, const SweepGeom &g, SplitPlan &p
     const long long lines = (long long)g.lines_a * g.lines_b;
     p.W = win + 1;
     p.x = g.pstride == 1;
+    p.after = ax.settled;
     if (d) {
         // float-float increments where kappa allows them, whatever the number
         // of lines

@@ -15,6 +15,7 @@
 #include "sscn_accum.cuh"
 #include "sscn_internal.h"
 #include "sscn_line.cuh"
+#include "sscn_pdl.cuh"
 
 namespace gp {
 namespace sp {
