@@ -13,6 +13,7 @@
 // coefficients are not symmetric, and the update is u = 2 v - psi with
 // (I - kappa T) v = psi.
 
+#include <algorithm>
 #include <cmath>
 #include <complex>
 #include <vector>
@@ -22,21 +23,15 @@
 #include "sscn_accum.cuh"
 #include "sscn_internal.h"
 #include "sscn_line.cuh"
+#include "sscn_rho.cuh"
 
 namespace gp {
 namespace {
 
 constexpr int kThreads = 64;                 // 2 warps, 16 lines per warp
 constexpr int kLinesPerBlock = kThreads / 2;
-constexpr int kPrefetchR = 4;
+constexpr int kAxialObsThreads = 128;
 constexpr unsigned kFull = 0xffffffffu;
-
-__device__ __forceinline__ double2 shfl16(double2 v)
-{
-    v.x = __shfl_xor_sync(kFull, v.x, 16);
-    v.y = __shfl_xor_sync(kFull, v.y, 16);
-    return v;
-}
 
 __device__ __forceinline__ double warp_sum(double v)
 {
@@ -61,9 +56,8 @@ __device__ double block_sum(double v, double *red)
     return r;
 }
 
-// Radial sweep of line k (z index) = psi[k * nr .. k * nr + nr - 1]; unknown
-// j = 1 .. m (m = nr) sits at stored index j - 1.  Top lane: j = 1 .. kmid-1,
-// bottom lane: j = m .. kmid+1, the top lane closes the middle row.
+// Radial sweep of line k (z index) = psi[k * nr .. k * nr + nr - 1], a lane pair
+// each.
 template <int MODE>
 __global__ void __launch_bounds__(kThreads)
 k_sweep_rho(double2 *__restrict__ psi, double2 *__restrict__ work, const RadialTables rt,
@@ -71,74 +65,13 @@ k_sweep_rho(double2 *__restrict__ psi, double2 *__restrict__ work, const RadialT
             const double2 *__restrict__ one, StepG sg, const double *__restrict__ scale)
 {
     const int lane = threadIdx.x & 31;
-    const bool top = lane < 16;
     const int line = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 16 + (lane & 15);
     const bool active = line < nz;
-    const int m = nr;
-    const int kmid = (m + 1) >> 1;
-    const int len = top ? kmid - 1 : m - kmid;
     const long long base = active ? (long long)line * nr : 0;
-    double2 *row = psi + base;
-    double2 *wl = work + base;
-    const double2 *cp = top ? rt.cp_top : rt.cp_bot;
-    const double2 *mult = top ? rt.mult_top : rt.mult_bot;
-    const double *kk = top ? rt.ka_top : rt.kc_bot;
     Calcnu<double, MODE> nl{};
     if (active) nl.setup(pr, pz, one, nullptr, nullptr, nullptr, line, 0, sg.value(), scale);
-    double2 d = make_double2(0.0, 0.0);
-    if (active) {
-        for (int t0 = 0; t0 < len; t0 += kPrefetchR) {
-            double2 pv[kPrefetchR];
-#pragma unroll
-            for (int q = 0; q < kPrefetchR; ++q)
-                if (t0 + q < len) pv[q] = row[top ? t0 + q : m - 1 - t0 - q];
-#pragma unroll
-            for (int q = 0; q < kPrefetchR; ++q) {
-                const int t = t0 + q;
-                if (t < len) {
-                    const int i = top ? t : m - 1 - t;
-                    const double2 p = nl.apply(pv[q], i);
-                    row[i] = p;
-                    d = LineOps<double, MODE>{kk[t]}.fwd(p, d, mult[t]);
-                    wl[i] = d;
-                }
-            }
-        }
-    }
-    const double2 other = shfl16(d);
-    double2 vk = make_double2(0.0, 0.0);
-    if (active && top) {
-        const int i = kmid - 1;
-        const double2 pk = nl.apply(row[i], i);
-        // kappa (a_k d'_{k-1} + c_k e_{k+1}) as kappa^ q with |kappa| folded into q
-        const double2 q = make_double2(fma(rt.ka_mid, d.x, rt.kc_mid * other.x),
-                                       fma(rt.ka_mid, d.y, rt.kc_mid * other.y));
-        vk = LineOps<double, MODE>{1.0}.fwd(pk, q, rt.mid);
-        row[i] = LineOps<double, MODE>::out(vk, pk);
-    }
-    const double2 vpair = shfl16(vk);
-    double2 v = top ? vk : vpair;
-    if (active) {
-        for (int t0 = len - 1; t0 >= 0; t0 -= kPrefetchR) {
-            double2 wv[kPrefetchR], lv[kPrefetchR];
-#pragma unroll
-            for (int q = 0; q < kPrefetchR; ++q)
-                if (t0 - q >= 0) {
-                    const int i = top ? t0 - q : m - 1 - t0 + q;
-                    wv[q] = wl[i];
-                    lv[q] = row[i];
-                }
-#pragma unroll
-            for (int q = 0; q < kPrefetchR; ++q) {
-                const int t = t0 - q;
-                if (t >= 0) {
-                    const int i = top ? t : m - 1 - t;
-                    v = LineOps<double, MODE>{0.0}.back(wv[q], cp[t], v);
-                    row[i] = LineOps<double, MODE>::out(v, lv[q]);
-                }
-            }
-        }
-    }
+    solve_rho<MODE>(psi + base, work + base, rt, nr, active, lane < 16, 16,
+                    [&](double2 p, int i) { return nl.apply(p, i); });
 }
 
 // calcnu of every point into pbuf (the radial windows overlap, so the
@@ -305,52 +238,74 @@ k_norm_partials_axial(const double2 *__restrict__ psi, int nr, long long count, 
     if (threadIdx.x == 0) partials[blockIdx.x] = r;
 }
 
-// One warp per line k; fixed-order per-lane sums, a warp tree, one row per line.
-__global__ void __launch_bounds__(256)
-k_observables_axial(const double2 *__restrict__ psi, ObsArgs a, double hr,
+// Observables: a thread walks `walk` values of z at one rho, so that the weights
+// rho, rho^2, V(rho) multiply its sums and not every point; the next line's value
+// is at hand for the z difference.  FP64-pipe bound: 15 FP64 instructions a point
+// (a warp per line with the weights at every point: 23, and too few warps).  1024
+// x 2048 with the finish: 142 us a warp per line, 107 here.  A block's sums in a
+// fixed order, one row each.
+__global__ void __launch_bounds__(kAxialObsThreads)
+k_observables_axial(const double2 *__restrict__ psi, ObsArgs a, double hr, int walk,
                     double *__restrict__ rows)
 {
-    const int lane = threadIdx.x & 31;
-    const long long line = (long long)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    __shared__ double part[kAxialObsThreads / 32][7];
     const int nr = a.nx, nz = a.ny;
-    if (line >= nz) return;
-    const int k = (int)line;
-    const double2 *row = psi + line * nr;
-    const bool has_z = k + 1 < nz;
-    double s0 = 0, sr = 0, sv = 0, s4 = 0, kr = 0, kz = 0;
-    for (int i = lane; i < nr; i += 32) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int k0 = blockIdx.y * walk, k1 = min(nz, k0 + walk);
+    double s[7] = {0, 0, 0, 0, 0, 0, 0};     // norm, r^2, z^2, V, |psi|^4, radial and axial differences
+    if (i < nr) {
+        const double2 *p = psi + (long long)k0 * nr + i;
+        const bool has_r = i + 1 < nr;
+        const double2 zero = make_double2(0.0, 0.0);
+        double2 v = *p;
+        double n = 0, z2 = 0, vz = 0, n2 = 0, kr = 0, kz = 0;
+#pragma unroll 4
+        for (int k = k0; k < k1; ++k, p += nr) {
+            const double2 nb = has_r ? p[1] : zero, up = k + 1 < nz ? p[nr] : zero;
+            const double am = fma(v.x, v.x, v.y * v.y);
+            n += am;
+            z2 = fma(a.y2[k], am, z2);
+            vz = fma(a.vy[k], am, vz);
+            n2 = fma(am, am, n2);
+            const double dx = nb.x - v.x, dy = nb.y - v.y;
+            kr = fma(dx, dx, fma(dy, dy, kr));
+            const double ex = up.x - v.x, ey = up.y - v.y;
+            kz = fma(ex, ex, fma(ey, ey, kz));
+            v = up;
+        }
         const double rho = (i + 0.5) * hr;
-        const double2 v = row[i];
-        const double am = fma(v.x, v.x, v.y * v.y);
-        const double w = rho * am;
-        s0 += w;
-        sr = fma(a.x2[i], w, sr);
-        sv = fma(a.vx[i], w, sv);
-        s4 = fma(w, am, s4);
-        const double2 nb = i + 1 < nr ? row[i + 1] : make_double2(0.0, 0.0);
-        const double dx = nb.x - v.x, dy = nb.y - v.y;
-        kr = fma(rho + 0.5 * hr, fma(dx, dx, dy * dy), kr);
-        const double2 nz_ = has_z ? row[i + nr] : make_double2(0.0, 0.0);
-        const double ex = nz_.x - v.x, ey = nz_.y - v.y;
-        kz = fma(rho, fma(ex, ex, ey * ey), kz);
+        s[0] = rho * n;
+        s[1] = a.x2[i] * s[0];
+        s[2] = rho * z2;
+        s[3] = fma(a.vx[i], s[0], rho * vz);
+        s[4] = rho * n2;
+        s[5] = (rho + 0.5 * hr) * kr;
+        s[6] = rho * kz;
     }
-    s0 = warp_sum(s0);
-    sr = warp_sum(sr);
-    sv = warp_sum(sv);
-    s4 = warp_sum(s4);
-    kr = warp_sum(kr);
-    kz = warp_sum(kz);
-    if (lane == 0) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int q = 0; q < 7; ++q) {
+        const double w = warp_sum(s[q]);
+        if (lane == 0) part[warp][q] = w;
+    }
+    __syncthreads();
+    if (threadIdx.x < 7) {
+        double w = 0.0;
+        for (int q = 0; q < (int)(blockDim.x >> 5); ++q) w += part[q][threadIdx.x];
+        part[0][threadIdx.x] = w;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
         const double sc = *a.scale, s2 = sc * sc;
-        double *out = rows + line * kObsWidth;
-        out[0] = s2 * s0;
-        out[1] = s2 * sr;
+        double *out = rows + (blockIdx.y * (long long)gridDim.x + blockIdx.x) * kObsWidth;
+        out[0] = s2 * part[0][0];
+        out[1] = s2 * part[0][1];
         out[2] = 0.0;
-        out[3] = s2 * a.y2[k] * s0;
-        out[4] = s2 * (sv + a.vy[k] * s0);
-        out[5] = s2 * s2 * s4;
-        out[6] = s2 * kr;
-        out[7] = s2 * kz;
+        out[3] = s2 * part[0][2];
+        out[4] = s2 * part[0][3];
+        out[5] = s2 * s2 * part[0][4];
+        out[6] = s2 * part[0][5];
+        out[7] = s2 * part[0][6];
         out[8] = 0.0;
     }
 }
@@ -386,6 +341,50 @@ void radial_tables(int m, double kre, double kim, double2 *cp_top, double2 *mult
     *mid = make_double2(f.real(), f.imag());
     *ka_mid = kabs * a(k);
     *kc_mid = kabs * c(k);
+}
+
+void radial_inc_tables(int m, double kre, double kim, float4 *top, float4 *bot, float4 *mid, int *win, int *near)
+{
+    using cd = std::complex<double>;
+    const cd kappa(kre, kim);
+    auto pack = [](cd v) {
+        const float rh = (float)v.real(), ih = (float)v.imag();
+        return make_float4(rh, ih, (float)(v.real() - rh), (float)(v.imag() - ih));
+    };
+    std::vector<cd> pt(m), pb(m);
+    std::vector<double> ft(m, 0.0), fb(m, 0.0);      // log2 of what a row passes on, in units of its rho
+    for (int i = 0; i < m; ++i) {
+        pt[i] = kappa / ((i + 0.5) * (1.0 + 2.0 * kappa) - (i ? kappa * (double)i * (double)i * pt[i - 1] : 0.0));
+        ft[i] = std::log2(std::abs(pt[i]) * (i + 1.0) * (i + 0.5) / (i + 1.5));
+        top[i] = pack(pt[i]);
+    }
+    for (int i = m - 1; i >= 0; --i) {
+        const double f = i + 1.0;
+        pb[i] = kappa / ((i + 0.5) * (1.0 + 2.0 * kappa) - (i < m - 1 ? kappa * f * f * pb[i + 1] : 0.0));
+        fb[i] = i ? std::log2(std::abs(pb[i]) * i * (i + 0.5) / (i - 0.5)) : 0.0;
+        bot[i] = pack(pb[i]);
+    }
+    for (int i = 0; i < m; ++i) {
+        const double f = i + 1.0;
+        mid[i] = pack(kappa / ((i + 0.5) * (1.0 + 2.0 * kappa) - (i ? kappa * (double)i * (double)i * pt[i - 1] : 0.0) -
+                               (i < m - 1 ? kappa * f * f * pb[i + 1] : 0.0)));
+    }
+    auto width = [&](double tol) {
+        for (int W = 1; W <= 64; ++W) {
+            bool ok = true;
+            double t = 0.0, b = 0.0;                 // sums over rows i - W + 1 .. i
+            for (int i = 0; i < m && ok; ++i) {
+                t += ft[i] - (i >= W ? ft[i - W] : 0.0);
+                b += fb[i] - (i >= W ? fb[i - W] : 0.0);
+                // a window of W whole rows: from row i - W + 1 up, from row i down
+                if (i >= W - 1) ok = t < tol && (i == W - 1 || b < tol);
+            }
+            if (ok) return W;
+        }
+        return 0;
+    };
+    *win = width(-55.0);
+    *near = width(-26.0);
 }
 
 void radial_window_tables(int m, double kre, double kim, int Lc, int W, double2 *cp, double2 *mult,
@@ -527,16 +526,25 @@ cudaError_t launch_norm_partials_axial(const void *psi, int nr, int nz, double h
     return cudaGetLastError();
 }
 
+// Lines a block walks: 16, fewer while there would be fewer than 8 blocks an SM.
+ObsWalk axial_obs_walk(int nr, int nz)
+{
+    ObsWalk w;
+    w.threads = std::min(kAxialObsThreads, (nr + 31) / 32 * 32);
+    const int cols = (nr + w.threads - 1) / w.threads;
+    w.walk = (int)std::min<long long>(16, std::max<long long>(2, (long long)cols * nz / (8 * 152)));
+    w.grid = dim3((unsigned)cols, (unsigned)((nz + w.walk - 1) / w.walk));
+    return w;
+}
+
 cudaError_t launch_observables_axial(const void *psi, const ObsArgs &a, double hr,
                                      double *scratch, double *sums, cudaStream_t st)
 {
-    const long long lines = a.ny;
-    double *rows = scratch, *stage = scratch + lines * kObsWidth;
-    const long long blocks = (lines * 32 + 255) / 256;
-    k_observables_axial<<<(unsigned)blocks, 256, 0, st>>>((const double2 *)psi, a, hr, rows);
+    const ObsWalk w = axial_obs_walk(a.nx, a.ny);
+    k_observables_axial<<<w.grid, w.threads, 0, st>>>((const double2 *)psi, a, hr, w.walk, scratch);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    return launch_rows_finish(rows, lines, stage, sums, st);
+    return launch_rows_finish(scratch, w.rows(), scratch + w.rows() * kObsWidth, sums, st);
 }
 
 }  // namespace gp

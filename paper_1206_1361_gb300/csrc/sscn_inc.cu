@@ -44,6 +44,7 @@
 // .. 2^93; a block that holds anything larger, or not finite, sweeps in FP64.
 
 #include "sscn_ff.cuh"
+#include "sscn_rho.cuh"
 #include "sscn_split.cuh"
 
 namespace gp {
@@ -70,10 +71,10 @@ struct IncArgs {
 
 constexpr unsigned kOff = (unsigned)(1023 - 127 - kLift) << 20;   // FP64 - FP32 exponent, lifted
 
-// Not finite, or too large for a lifted float.
-__device__ __forceinline__ bool too_large(double x)
+// Not finite, or too large for a lifted float (MARGIN: times 2^MARGIN).
+template <int MARGIN = 0> __device__ __forceinline__ bool too_large(double x)
 {
-    return ((unsigned)__double2hiint(x) & 0x7fffffffu) >= kOff + (250u << 20);
+    return ((unsigned)__double2hiint(x) & 0x7fffffffu) >= kOff + ((250u - MARGIN) << 20);
 }
 
 // 2^kLift x as a float-float pair: hi the nearest float (ties away from zero),
@@ -314,11 +315,130 @@ template <int MODE> struct IncLane : HalfLine {
     }
 };
 
+// ------------------------------------------------------------------ radial
+//
+// The radial operator of the axially symmetric form, rows i = 0 .. m - 1, times
+// rho_i / h = i + 1/2, is the difference of the fluxes i (psi_i - psi_{i-1})
+// through the faces either side: symmetric, its couplings whole numbers that
+// float-float products take exactly.  As above with (face f between a row and
+// the one its half came from, f' the face ahead, p the row's coefficient in
+// radial_inc_tables):
+//     S = f' (psi_{t+1} - psi_t) - f (psi_t - psi_{t-1})
+//     e_t = S + f p_{t-1} e_{t-1},   g_k = p_k (S_k + both carries)
+//     g_t = p_t (e_t + f' g_{t+1}),  2 Delta_t = 2 g_t
+struct RadArgs {
+    SplitArgs<double> s;
+    int near;
+    const float4 *mid;
+    double2 *work;
+    RadialTables rt;
+};
+
+constexpr int kRadialBits = 15;          // S and e are at most 2^15 times psi
+
+__device__ __forceinline__ FC ntimes(FC z, float n) { return ff::lmul(z, f2(n, n), f2(0.f, 0.f)); }
+__device__ __forceinline__ FfCoef expand(float4 v) { return FfCoef{f2(v.x, v.x), f2(v.z, v.z), f2(-v.y, v.y), f2(-v.w, v.w)}; }
+
+// both coefficient tables of m rows in shared memory
+__host__ __device__ __forceinline__ size_t rad_table_bytes(int m) { return (size_t)2 * (slot_of(m) + 1) * sizeof(float4); }
+
+template <int MODE> struct RadLane : HalfLine {
+    const RadArgs &A;
+    const float4 *tab;
+
+    __device__ __forceinline__ RadLane(const RadArgs &args, const float4 *tables, int seg)
+        : HalfLine(args.s.n, args.s.S, args.s.W, seg), A(args), tab(tables + (top ? 0 : slot_of(m) + 1))
+    {
+    }
+    __device__ __forceinline__ float face(int t) const { return (float)(top ? t : m - t); }
+    __device__ __forceinline__ FfCoef p(int t) const
+    {
+        t = max(t, 0);                   // (before the first row: its carry is zero)
+        return expand(tab[slot_of(top ? t : m - 1 - t)]);
+    }
+
+    // As IncLane::solve<true>.
+    template <typename Ld, typename Out> __device__ __forceinline__ void solve(bool active, Ld ld, Out out) const
+    {
+        FC e = ff::cz(), ev[kIncP], cur = ff::cz(), d0 = ff::cz();
+        const float f0 = face(to), ahead = top ? 1.f : -1.f;       // the faces in the direction of t
+        if (active) {
+            int t = ts;
+            const int t1 = max(ts, to - A.near);
+            if (t < t1) {
+                float2 ee = f2(0.f, 0.f);
+                const FC a0 = ld(row(t - 1));
+                FC a1 = ld(row(t));
+                float f = face(t);
+                float2 dd = ff::mul(f2(f, f), ff::add(ff::sub(a1.hi, a0.hi), ff::sub(a1.lo, a0.lo)));
+                for (; t < t1; ++t) {
+                    const FC a2 = ld(row(t + 1));
+                    const float fn = face(t + 1);
+                    const float2 dn = ff::mul(f2(fn, fn), ff::add(ff::sub(a2.hi, a1.hi), ff::sub(a2.lo, a1.lo)));
+                    const FfCoef k = p(t - 1);
+                    const float2 q = ff::mul(f2(f, f), ee);
+                    float2 s = ff::sub(dn, dd);
+                    s = ff::fma2(q, k.rh, s);
+                    if (MODE != 0) s = ff::fma2(ff::swap(q), k.ih, s);
+                    ee = s;
+                    dd = dn;
+                    a1 = a2;
+                    f = fn;
+                }
+                e.hi = ee;
+            }
+            cur = ld(row(t));
+            d0 = ntimes(ff::sub(cur, ld(row(t - 1))), face(t));
+            auto rhs = [&](int at, float f) {
+                const FC next = ld(row(at + 1)), d1 = ntimes(ff::sub(next, cur), f), s = ff::sub(d1, d0);
+                cur = next;
+                d0 = d1;
+                return s;
+            };
+            for (float f = face(t); t < to; ++t, f += ahead)
+                e = ff::add(rhs(t, f + ahead), ntimes(rtimes<MODE>(e, p(t - 1)), f));
+#pragma unroll
+            for (int q = 0; q < kIncP; ++q)
+                if (to + q <= te)
+                    ev[q] = e = ff::add(rhs(to + q, fmaf(q + 1, ahead, f0)),
+                                        ntimes(rtimes<MODE>(e, p(to + q - 1)), fmaf(q, ahead, f0)));
+        }
+        const FC c = ntimes(rtimes<MODE>(e, p(te)), face(kt));
+        FC o;
+        o.hi.x = __shfl_xor_sync(0xffffffffu, c.hi.x, 1);
+        o.hi.y = __shfl_xor_sync(0xffffffffu, c.hi.y, 1);
+        o.lo.x = __shfl_xor_sync(0xffffffffu, c.lo.x, 1);
+        o.lo.y = __shfl_xor_sync(0xffffffffu, c.lo.y, 1);
+        FC g = ff::cz();
+        if (active && top) {
+            const FC next = ld(row(kt + 1)), s = ff::sub(ntimes(ff::sub(next, cur), face(kt + 1)), d0);
+            g = rtimes<MODE>(ff::add(ff::add(s, c), o), expand(__ldg(A.mid + kt)));
+        }
+        __syncthreads();
+        if (active && top) out(row(kt), g);
+        FC w;
+        w.hi.x = __shfl_xor_sync(0xffffffffu, g.hi.x, 1);
+        w.hi.y = __shfl_xor_sync(0xffffffffu, g.hi.y, 1);
+        w.lo.x = __shfl_xor_sync(0xffffffffu, g.lo.x, 1);
+        w.lo.y = __shfl_xor_sync(0xffffffffu, g.lo.y, 1);
+        if (!top) g = w;
+        if (active) {
+#pragma unroll
+            for (int q = kIncP - 1; q >= 0; --q)
+                if (to + q <= te) {
+                    g = rtimes<MODE>(ff::add(ev[q], ntimes(g, fmaf(q + 1, ahead, f0))), p(to + q));
+                    out(row(to + q), g);
+                }
+        }
+    }
+};
+
 // ----------------------------------------------------------------- kernels
 
 // Resident blocks the kernels are compiled for: 3 of 256 threads (80 registers
-// a thread).
-template <int THREADS> constexpr int kMinBlocks = THREADS == 256 ? 3 : 1;
+// a thread), or 2 of 512 (64; lines of more than 1024 rows: the z sweep of an
+// axial 1024 x 2048 took 62 us with one, 52 with two).
+template <int THREADS> constexpr int kMinBlocks = THREADS == 256 ? 3 : 2;
 
 // x sweep: as k_split_x, thread (row, seg) moving the row's points seg, seg + 2 S,
 // ...  A point's calcnu goes back to memory and is read again (from L1 or L2)
@@ -498,6 +618,87 @@ __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_yz(const _
     }
 }
 
+// Radial sweep: as k_inc_x (NL), stored point i of a line being row i + 1.
+// Measured at 1024 x 2048, real time: 73 us (the segmented windows, with calcnu
+// as a pass of its own: 175).  The potential's two complex products, 8 FP64
+// instructions a point, hold the FP64 pipe 27 us of it; the rest is issue slots
+// and the latency of blocks of two lines (three resident an SM, next to 36 KB of
+// coefficients each).
+template <int MODE, int THREADS>
+__global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_rho(const __grid_constant__ RadArgs A)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ double g_of_step;
+    __shared__ float2 g_lifted;
+    const SplitArgs<double> &a = A.s;
+    const int n = a.n, m = n - 1, pitch = slot_of(n) + 1;
+    float4 *coef = reinterpret_cast<float4 *>(smem_raw);
+    Calcnu<double, MODE> *row_nl = reinterpret_cast<Calcnu<double, MODE> *>(smem_raw + rad_table_bytes(m));
+    float4 *tile = reinterpret_cast<float4 *>(row_nl + a.per);
+    const int line0 = blockIdx.x * a.per;
+    const int rows = min(a.per, a.lines_a - line0);
+    const int lanes = 2 * a.S;
+    const int q = threadIdx.x / lanes, seg = threadIdx.x - q * lanes;
+    const bool active = q < rows;
+    const int at = (active ? q : 0) * pitch;
+    double2 *row = a.psi + (long long)(line0 + (active ? q : 0)) * m;
+    for (int i = threadIdx.x; i < m; i += blockDim.x) {
+        coef[slot_of(i)] = A.rt.inc_top[i];
+        coef[slot_of(m) + 1 + slot_of(i)] = A.rt.inc_bot[i];
+    }
+    for (int r = threadIdx.x; r < a.per; r += blockDim.x)
+        tile[r * pitch] = tile[r * pitch + slot_of(n)] = make_float4(0.f, 0.f, 0.f, 0.f);
+    pdl_wait();
+    double2 v[kIncP];
+    if (active) {
+#pragma unroll
+        for (int b = 0; b < kIncP; ++b) {
+            const int i = seg + b * lanes;
+            if (i < m) v[b] = row[i];
+        }
+    }
+    if (threadIdx.x == 0) {
+        const double G = a.sg.value(), sc = MODE == 0 && a.scale ? *a.scale : 1.0;
+        g_of_step = G * sc * sc;
+        g_lifted = lifted_g(G * sc * sc);
+    }
+    for (int r = threadIdx.x; r < rows; r += blockDim.x)
+        row_nl[r].setup(a.px, a.py, a.pz, nullptr, nullptr, nullptr, line0 + r, 0, 0.0, a.scale);
+    __syncthreads();                         // row_nl, G
+    bool big = false;
+    if (active) {
+        const double G = g_of_step;
+        const float2 gl = g_lifted;
+#pragma unroll
+        for (int b = 0; b < kIncP; ++b) {
+            const int i = seg + b * lanes;
+            if (i < m) {
+                v[b] = calcnu_at<MODE, false>(v[b], row_nl[q], i, make_double2(0.0, 0.0), gl, G);
+                row[i] = v[b];
+                big = big || too_large<kRadialBits>(v[b].x) || too_large<kRadialBits>(v[b].y);
+                tile[at + slot_of(i + 1)] = pack(lift(v[b]));
+            }
+        }
+    }
+    if (__syncthreads_or(big)) {
+        const long long base = (long long)(line0 + (active ? q : 0)) * m;
+        solve_rho<MODE>(a.psi + base, A.work + base, A.rt, m, active && seg < 2, seg == 0, 1,
+                        [](double2 p, int) { return p; });
+        return;
+    }
+    const RadLane<MODE> lane(A, coef, active ? seg : (threadIdx.x & 1));
+    lane.solve(active, [&](int i) { return unpack(tile[at + slot_of(i)]); },
+               [&](int i, FC g) { tile[at + slot_of(i)] = pack(g); });
+    __syncthreads();
+    if (active) {
+#pragma unroll
+        for (int b = 0; b < kIncP; ++b) {
+            const int i = seg + b * lanes;
+            if (i < m) row[i] = plus<1, true>(row[i], unpack(tile[at + slot_of(i + 1)]));
+        }
+    }
+}
+
 template <int MODE, bool NL, bool P3> cudaError_t go_x(const SplitPlan &p, const IncArgs &a, cudaStream_t st)
 {
     auto kern = p.threads <= 256 ? k_inc_x<MODE, NL, P3, 256> : k_inc_x<MODE, NL, P3, kSplitThreads>;
@@ -516,6 +717,56 @@ cudaError_t go_yz(const SplitPlan &p, const IncArgs &a, cudaStream_t st)
 }
 
 }  // namespace
+
+bool rho_inc_plan(const RadialTables &rt, int nr, int nz, SplitPlan &p)
+{
+    p = SplitPlan{};
+    if (rt.win < 1 || rt.near < 1 || rt.kre > kIncKappaImag || rt.kim > kIncKappaReal) return false;
+    const size_t tables = rad_table_bytes(nr);
+    const size_t row = (size_t)(slot_of(nr + 1) + 1) * sizeof(float4) + sizeof(Calcnu<double, 0>);
+    p.P = kIncP;
+    p.S = (nr + 2 * kIncP - 1) / (2 * kIncP);
+    p.W = rt.win + 1;
+    p.x = p.increment = p.after = true;
+    const int lanes = 2 * p.S;
+    if (lanes > kSplitThreads || tables + row > kSplitSmem) return false;
+    // as the x sweep: about 256 lanes and at most 64 KB of rows
+    int per = lanes >= 256 ? 1 : 256 / lanes;
+    while (per > 1 && per * row > 64 * 1024) --per;
+    if (nz < kSms * per) per = (nz + kSms - 1) / kSms;
+    p.per = per;
+    p.smem = tables + per * row;
+    p.grid_x = (unsigned)((nz + per - 1) / per);
+    p.grid_y = 1;
+    p.threads = (per * lanes + 31) / 32 * 32;
+    return true;
+}
+
+cudaError_t launch_sweep_rho_inc(const SplitPlan &p, int mode, void *psi, void *work, const RadialTables &rt,
+                                 int nr, int nz, const NonlinArgs &nl, cudaStream_t st)
+{
+    RadArgs a{};
+    a.s.psi = static_cast<double2 *>(psi);
+    a.s.n = nr + 1;
+    a.s.S = p.S;
+    a.s.W = p.W;
+    a.s.per = p.per;
+    a.s.lines_a = nz;
+    a.s.px = nl.px;
+    a.s.py = nl.py;
+    a.s.pz = nl.pz;
+    a.s.sg = nl.g;
+    a.s.scale = nl.scale;
+    a.near = rt.near + 1;
+    a.mid = rt.inc_mid;
+    a.work = static_cast<double2 *>(work);
+    a.rt = rt;
+    auto kern = p.threads <= 256 ? (mode == 0 ? k_inc_rho<0, 256> : k_inc_rho<1, 256>)
+                                 : (mode == 0 ? k_inc_rho<0, kSplitThreads> : k_inc_rho<1, kSplitThreads>);
+    cudaError_t e = allow_smem(kern, p.smem);
+    if (e != cudaSuccess) return e;
+    return launch_after(p.after, kern, p.grid_x, p.threads, p.smem, st, a);
+}
 
 bool inc_applies(const AxisTables &ax) { return ax.kre <= kIncKappaImag && ax.kim <= kIncKappaReal; }
 

@@ -288,6 +288,7 @@ struct ObsWalk {
     long long rows() const { return (long long)grid.x * grid.y * grid.z; }
 };
 ObsWalk obs_walk(int prec, int nx, int ny, int nz);
+ObsWalk axial_obs_walk(int nr, int nz);
 cudaError_t launch_observables(int prec, const void *psi, const ObsArgs &a,
                                double *scratch, double *sums, cudaStream_t st);
 // Fixed-order finish of `rows` partials rows of kObsWidth doubles into sums: one
@@ -316,6 +317,10 @@ struct RadialTables {
     const double *ka_top = nullptr, *kc_bot = nullptr;
     double2 mid{0, 0};
     double ka_mid = 0, kc_mid = 0;
+    // The increment sweep (radial_inc_tables; win = 0: it does not apply)
+    double kre = 0, kim = 0;
+    const float4 *inc_top = nullptr, *inc_bot = nullptr, *inc_mid = nullptr;
+    int win = 0, near = 0;
 };
 // Host computation of those tables for kappa = kre + i kim (kre or kim zero).
 void radial_tables(int m, double kre, double kim, double2 *cp_top, double2 *mult_top,
@@ -326,6 +331,22 @@ void radial_tables(int m, double kre, double kim, double2 *cp_top, double2 *mult
 // by the line), nl.pz = a one-entry table (1, 0).
 cudaError_t launch_sweep_rho(int mode, void *psi, void *work, const RadialTables &rt, int nr,
                              int nz, const NonlinArgs &nl, cudaStream_t st);
+
+
+// Radial sweep of every line whose increment is computed in float-float
+// (sscn_inc.cu).  Host: its coefficients, rows i = 0 .. m - 1 (m entries each)
+// as float-float complex numbers (hi re, hi im, lo re, lo im): with rho_i = i +
+// 1/2,
+//   top[i] = kappa / ((1 + 2 kappa) rho_i - kappa i^2 top[i-1])
+//   bot[i] = kappa / ((1 + 2 kappa) rho_i - kappa (i+1)^2 bot[i+1])
+//   mid[i]: both terms
+// and the rows over which a carry is damped below 2^-55 (win, 0: more than 64)
+// and 2^-26 (near).
+void radial_inc_tables(int m, double kre, double kim, float4 *top, float4 *bot, float4 *mid, int *win, int *near);
+// False if the sweep does not apply (kappa, the line's length).
+bool rho_inc_plan(const RadialTables &rt, int nr, int nz, SplitPlan &plan);
+cudaError_t launch_sweep_rho_inc(const SplitPlan &plan, int mode, void *psi, void *work, const RadialTables &rt,
+                                 int nr, int nz, const NonlinArgs &nl, cudaStream_t st);
 
 // Segmented-window sweeps of the axial form (few, long lines).  Each line is
 // cut into cores of Lc unknowns; a thread solves its core's rows extended by
@@ -372,7 +393,7 @@ cudaError_t launch_zero_axial(void *psi, int nr, cudaStream_t st);
 // FP64 sums of rho_i |psi|^2 into `blocks` partials.
 cudaError_t launch_norm_partials_axial(const void *psi, int nr, int nz, double hr,
                                        const Partials &out, int blocks, cudaStream_t st);
-// Observables rows (one per line k): S0 = sum rho |psi|^2, sum rho^3 |psi|^2,
+// Observables rows (one per block of axial_obs_walk): S0 = sum rho |psi|^2, sum rho^3 |psi|^2,
 // 0, z^2 S0, sum rho V |psi|^2, sum rho |psi|^4, sum rho_{i+1/2} |psi_{i+1} - psi_i|^2,
 // sum rho |psi_{k+1} - psi_k|^2, 0 (times the pending scale), then the finish.
 // a.x2 / a.vx: rho^2 and gamma^2 rho^2 / 2; a.y2 / a.vy: z^2 and lambda^2 z^2 / 2.

@@ -15,6 +15,7 @@
 // given launch shape always produces the same bits (the observables do not
 // depend on the launch shape at all: one partials row per grid line).
 
+#include <algorithm>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -802,7 +803,7 @@ long long obs_stage_rows(long long rows)
 long long obs_scratch_doubles(const ObsArgs &a)
 {
     long long rows = obs_walk(kC128, a.nx, a.ny, a.nz).rows();      // the most of any precision
-    if (a.nz == 1 && a.ny > rows) rows = a.ny;      // the axial form: a row per line
+    if (a.nz == 1) rows = std::max(rows, axial_obs_walk(a.nx, a.ny).rows());
     return (rows + obs_stage_rows(rows)) * kObsWidth;
 }
 

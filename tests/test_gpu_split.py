@@ -214,3 +214,46 @@ def test_batch_launch_forms_agree_bit_for_bit(prec):
     for a, c in zip(got[0][0], got[1][0]):
         assert np.array_equal(a, c)
     assert got[0][1] == got[1][1]
+
+
+def axial_run(nr, nz, kappa, g, mode, psi0, steps, path=gp.GP_PATH_AUTO, strang=False):
+    dt = 1e-3
+    h = (dt / (4.0 * kappa)) ** 0.5
+    with gp.Solver.axial(nr, nz, h, 1.1 * h, dt, 1.0, 2.0, g, mode) as s:
+        s.set_path(path)
+        if strang:
+            s.set_splitting(gp.GP_SPLIT_STRANG).set_modulation(3.0, 40.0)
+        return s.load(psi0).step(steps).psi()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("nr,nz", [(3, 3), (16, 40), (17, 33), (49, 18), (256, 130), (1023, 301), (1500, 35), (21, 2048),
+                                   (3700, 4), (5000, 4), (24, 2300)])
+@pytest.mark.parametrize("mode,kappa", [(gp.GP_IMAG, 0.004), (gp.GP_IMAG, 0.024), (gp.GP_REAL, 0.0125), (gp.GP_REAL, 0.059)])
+@pytest.mark.parametrize("strang", [False, True])
+def test_axial_increment_sweeps_match_the_oracle(nr, nz, mode, kappa, strang):
+    """The radial increment sweep (and the axial one) at every remainder of the
+    cut, at the longest lines it takes and past them."""
+    require_gpu()
+    dt, g, steps = 1e-3, 5.0, 5
+    h = (dt / (4.0 * kappa)) ** 0.5
+    psi0 = rand_state((nr, nz, 1), 5)[0]
+    psi0[1:, 0] = psi0[1:, -1]                        # (the axis rho = h / 2 is a live row)
+    got = axial_run(nr, nz, kappa, g, mode, psi0, steps, strang=strang)
+    par = oracle.AxialParams.make(nr, nz, h, 1.1 * h, dt, 1.0, 2.0, g, mode)
+    want = oracle.axial_step(par, psi0.copy(), steps, 0, True, 3.0, 40.0) if strang else oracle.axial_step(par, psi0.copy(), steps)
+    assert rel_l2(got, want) <= 1e-12
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("scale", [2.0 ** -300, 2.0 ** 77, 2.0 ** 79, 2.0 ** 92, 2.0 ** 400])
+def test_axial_values_beyond_the_lifted_floats(scale):
+    """Linear real-time steps scale exactly by powers of two: large values take
+    the FP64 branch, tiny ones lose only what is far below the largest."""
+    require_gpu()
+    nr, nz = 100, 70
+    psi0 = rand_state((nr, nz, 1), 6)[0]
+    want = axial_run(nr, nz, 0.02, 0.0, gp.GP_REAL, psi0, 3, path=gp.GP_PATH_EXACT)
+    got = axial_run(nr, nz, 0.02, 0.0, gp.GP_REAL, psi0 * scale, 3) / scale
+    # below the lifted range the increment is dropped: up to 8 kappa per sweep
+    assert rel_l2(got, want) <= (1e-12 if scale > 1e-30 else 3 * 2 * 8 * 0.02)
