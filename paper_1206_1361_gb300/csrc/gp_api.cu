@@ -551,6 +551,21 @@ bool prefers_split(const gp_ctx *c, int axis)
     return 8.0 + std::max(0.06 * n, p / 370e3) > 4.0 + p / 210e3;
 }
 
+// The same for the float-float form, whose TMA pipeline walks a line at 0.42 us
+// a row on x and 0.17 on y and z.  Measured on GB300 (us; n rows a line, p
+// points): TMA max(10 + 0.42 n, 10 + p / 80e3) on x, 8 + max(0.17 n, p / 150e3)
+// on y and z; sub-lines 12 + p / 53e3 and 8 + p / 100e3 (the windows' extra rows).
+// 500 x 384: 233 and 76 against 19 and 13; 64^3: 40, 21, 20 against 19, 11, 10;
+// 512 x 128 x 128, x: 261 against 167; 256^3 stays: 246, 127, 123 against 319,
+// 182, 177.
+bool prefers_ff_split(const gp_ctx *c, int axis)
+{
+    if (c->path_opt != GP_PATH_AUTO || c->tile_shape != 0) return false;
+    const double n = edge(c->grid, axis), p = (double)points(c->grid);
+    if (axis == 0) return 10.0 + std::max(0.42 * n, p / 80e3) > 12.0 + p / 53e3;
+    return std::max(0.17 * n, p / 150e3) > p / 100e3;
+}
+
 // Axial form: both sweeps with float-float increments, in place, unless the
 // exact path was chosen.  Otherwise the segmented windows (or the exact path)
 // take both.  1024 x 2048 real time, us: 73 + 52 against 175 + 80 in windows; 64 x
@@ -591,6 +606,11 @@ cudaError_t launch_sweep(gp_ctx *c, int axis, const gp::NonlinArgs *nl, bool nl_
             fn.pz = nl->pz;
             fn.g = nl->g;
             fn.scale = nl->scale;
+        }
+        gp::SplitPlan plan;
+        if (prefers_ff_split(c, axis) && gp::split_plan(GP_C128, ax, g, plan) && plan.increment) {
+            if (blocks) *blocks = gp::split_blocks(plan);
+            return gp::launch_sweep_ffinc(plan, c->mode, c->psi, ax, g, nl ? &fn : nullptr, norm, c->stream);
         }
         if (blocks) *blocks = gp::ff_blocks(c->tile_shape, g);
         return gp::launch_sweep_ff(c->tile_shape, c->mode, axis, c->maps[axis], c->ffax[c->mode][axis],

@@ -183,5 +183,69 @@ __device__ __forceinline__ K expand(double re, double im)
     return K{f2(r.x, r.x), f2(r.y, r.y), f2(-i.x, i.x), f2(-i.y, i.y)};
 }
 
+// calcnu at one point of an x line (sscn_ff.cu).
+template <int MODE> struct FfRow {
+    FfCoef pyz;          // P_y[j] P_z[k] (times s in imaginary time), expanded
+    float2 acoef;        // G (times s^2 in imaginary time)
+    float2 fyz;          // imaginary time: s P_y[j] P_z[k] as a scalar pair
+
+    // the line's factors (G, the pending scale: of the step)
+    __device__ __forceinline__ void setup(double2 y, double2 z, double G, double s)
+    {
+        if (MODE == 0) {
+            const double f = s * y.x * z.x;
+            fyz = split(f);
+            acoef = split(G * s * s);
+            pyz = expand(f, 0.0);
+        } else {
+            pyz = expand(y.x * z.x - y.y * z.y, y.x * z.y + y.y * z.x);
+            acoef = split(G);
+            fyz = f2(0.f, 0.f);
+        }
+    }
+
+    // x: the factor along the line at the point
+    __device__ __forceinline__ C apply(C p, const FfCoef &x) const
+    {
+        const float2 a = s_mul(acoef, abs2(p));
+        if (MODE == 0) {
+            // eps = exp(-a) - 1 = -a + a^2/2 - a^3/6 + a^4/24 - a^5/120 + ...
+            float2 eps;
+            if (fabsf(a.x) < 0x1p-8f) {
+                const float q = __fmul_rn(a.x, a.x);
+                float qe = fmaf(a.x, a.x, -q);
+                qe = fmaf(2.f * a.x, a.y, qe);
+                eps = s_two_sum(-a.x, 0.5f * q);
+                const float tail = fmaf(q, fmaf(a.x, -1.f / 120, 1.f / 24) * q, -a.x * q * (1.f / 6));
+                eps = s_norm(f2(eps.x, eps.y + ((0.5f * qe - a.y) + tail)));
+            } else {
+                eps = split(expm1(-join(a)));
+            }
+            const float2 f = s_mul(fyz, f2(x.rh.x, x.rl.x));
+            const float2 F = s_norm(s_add(f, s_mul(f, eps)));
+            return norm(lmul(p, f2(F.x, F.x), f2(F.y, F.y)));
+        }
+        // delta = exp(-i a) - 1 = (cos a - 1) - i sin a
+        float2 dr, di;
+        if (fabsf(a.x) < 0x1p-8f) {
+            const float q = __fmul_rn(a.x, a.x);
+            float qe = fmaf(a.x, a.x, -q);
+            qe = fmaf(2.f * a.x, a.y, qe);
+            // cos a - 1 = -a^2/2 + a^4/24 - ...   (a^6/720 < 2^-57)
+            dr = f2(-0.5f * q, fmaf(q * q, 1.f / 24, -0.5f * qe));
+            // -sin a = -a + a^3/6 - a^5/120 + ...  (a^7/5040 < 2^-68)
+            di = f2(-a.x, fmaf(a.x * q, fmaf(q, -1.f / 120, 1.f / 6), -a.y));
+        } else {
+            double sh, ch;
+            sincos(0.5 * join(a), &sh, &ch);
+            dr = split(-2.0 * sh * sh);
+            di = split(-2.0 * sh * ch);
+        }
+        const FfCoef D{f2(dr.x, dr.x), f2(dr.y, dr.y), f2(-di.x, di.x), f2(-di.y, di.y)};
+        const C q2 = cmul(cmul(p, x), pyz);
+        return norm(add(q2, cmul(q2, D)));
+    }
+};
+
 }  // namespace ff
 }  // namespace gp

@@ -618,6 +618,126 @@ __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_yz(const _
     }
 }
 
+// The float-float form (psi itself a pair): as k_inc_x and k_inc_yz, without the
+// conversions.  Nothing here is too large for the lifted form's range that calcnu
+// or the norm, which square psi in FP32, would not lose as well.
+struct FfIncArgs {
+    IncArgs i;
+    const FfCoef *px;
+};
+
+__device__ __forceinline__ FC plus_twice(FC p, FC g)
+{
+    const float2 two = f2(2.f, 2.f);
+    return ff::norm(ff::add(p, FC{ff::mul(two, g.hi), ff::mul(two, g.lo)}));
+}
+
+template <int MODE, bool NL, int THREADS>
+__global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_ffinc_x(const __grid_constant__ FfIncArgs F)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const IncArgs &A = F.i;
+    const SplitArgs<double> &a = A.s;
+    const int n = a.n, pitch = slot_of(n) + 1;
+    ff::FfRow<MODE> *row_nl = reinterpret_cast<ff::FfRow<MODE> *>(smem_raw + inc_coef_bytes(a.conv));
+    static_assert(sizeof(ff::FfRow<MODE>) <= sizeof(Calcnu<double, 0>), "the plan's bytes a row");
+    float4 *tile = reinterpret_cast<float4 *>(row_nl + a.per);
+    const int line0 = blockIdx.x * a.per;
+    const int rows = min(a.per, a.lines_a * a.lines_b - line0);
+    const int lanes = 2 * a.S;
+    const int q = threadIdx.x / lanes, seg = threadIdx.x - q * lanes;
+    const bool active = q < rows;
+    const int at = (active ? q : 0) * pitch;
+    float4 *row = reinterpret_cast<float4 *>(a.psi) + (long long)(line0 + (active ? q : 0)) * n;
+    stage_inc<MODE>(A, smem_raw);
+    for (int r = threadIdx.x; r < a.per; r += blockDim.x)
+        tile[r * pitch] = tile[r * pitch + slot_of(n)] = make_float4(0.f, 0.f, 0.f, 0.f);
+    pdl_wait();
+    float4 v[kIncP];
+    if (active) {
+#pragma unroll
+        for (int b = 0; b < kIncP; ++b) {
+            const int i = 1 + seg + b * lanes;
+            if (i < n) v[b] = row[i];
+        }
+    }
+    if (NL) {
+        for (int r = threadIdx.x; r < rows; r += blockDim.x) {
+            const int L = line0 + r;
+            row_nl[r].setup(a.py[L % a.lines_a], a.pz[L / a.lines_a], a.sg.value(),
+                            MODE == 0 && a.scale ? *a.scale : 1.0);
+        }
+        __syncthreads();
+    }
+    if (active) {
+#pragma unroll
+        for (int b = 0; b < kIncP; ++b) {
+            const int i = 1 + seg + b * lanes;
+            if (i < n) {
+                if constexpr (NL) {
+                    v[b] = pack(row_nl[q].apply(unpack(v[b]), F.px[i]));
+                    row[i] = v[b];
+                }
+                tile[at + slot_of(i)] = v[b];
+            }
+        }
+    }
+    __syncthreads();
+    const IncLane<MODE> lane(A, smem_raw, active ? seg : (threadIdx.x & 1));
+    lane.template solve<true>(
+        active, 1, [&](int i) { return unpack(tile[at + slot_of(i)]); },
+        [&](int, int i, FC g) { tile[at + slot_of(i)] = pack(g); });
+    __syncthreads();
+    if (active) {
+#pragma unroll
+        for (int b = 0; b < kIncP; ++b) {
+            const int i = 1 + seg + b * lanes;
+            if (i < n) row[i] = pack(plus_twice(unpack(row[i]), unpack(tile[at + slot_of(i)])));
+        }
+    }
+}
+
+template <int MODE, bool NORM, int THREADS>
+__global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_ffinc_yz(const __grid_constant__ FfIncArgs F)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ double red[32];
+    const IncArgs &A = F.i;
+    const SplitArgs<double> &a = A.s;
+    float4 *tile = reinterpret_cast<float4 *>(smem_raw + inc_coef_bytes(a.conv));
+    const int n = a.n, XL = a.per;
+    const int xl = threadIdx.x & (XL - 1), seg = threadIdx.x / XL;
+    const int la = blockIdx.x * XL + xl, lb = blockIdx.y;
+    const bool active = la < a.lines_a && seg < 2 * a.S;
+    const IncLane<MODE> lane(A, smem_raw, seg < 2 * a.S ? seg : (seg & 1));
+    float4 *line = reinterpret_cast<float4 *>(a.psi) + (active ? (long long)la * a.stride_a + (long long)lb * a.stride_b : 0);
+    stage_inc<MODE>(A, smem_raw);
+    pdl_wait();
+    auto at_of = [&](int i) { return slot_of(i) * XL + xl; };
+    if (active) {
+        float4 p[kIncP];
+#pragma unroll
+        for (int q = 0; q < kIncP; ++q)
+            if (lane.first + q <= lane.last) p[q] = line[(long long)lane.row(lane.first + q) * a.pstride];
+#pragma unroll
+        for (int q = 0; q < kIncP; ++q)
+            if (lane.first + q <= lane.last) tile[at_of(lane.row(lane.first + q))] = p[q];
+        if (seg == 0) tile[at_of(0)] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (seg == 1) tile[at_of(n)] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    __syncthreads();
+    float2 acc = f2(0.f, 0.f);
+    lane.template solve<false>(
+        active, XL, [&](int i) { return unpack(tile[at_of(i)]); },
+        [&](int, int i, FC g) {
+            const FC u = plus_twice(unpack(tile[at_of(i)]), g);
+            line[(long long)i * a.pstride] = pack(u);
+            if (NORM) acc = ff::s_add(acc, ff::abs2(u));
+        });
+    if (NORM)
+        block_partial(active ? ff::join(acc) : 0.0, red, &a.partials[(long long)blockIdx.y * gridDim.x + blockIdx.x]);
+}
+
 // Radial sweep: as k_inc_x (NL), stored point i of a line being row i + 1.
 // Measured at 1024 x 2048, real time: 73 us (the segmented windows, with calcnu
 // as a pass of its own: 175).  The potential's two complex products, 8 FP64
@@ -699,6 +819,23 @@ __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_rho(const 
     }
 }
 
+IncArgs inc_args(const SplitPlan &p, int mode, void *psi, const AxisTables &ax, const SweepGeom &g,
+                 const NonlinArgs *nl, const Partials *norm_out)
+{
+    IncArgs a{};
+    a.s = split_args<kFp64>(p, mode, psi, ax, g, nl, norm_out);
+    a.rinf = ff_expand(a.s.rinf);
+    for (int q = 0; q < kIncEnds; ++q) {
+        const double2 f = a.s.mid[q];
+        a.kmid[q] = ff_expand(mode == 0 ? make_double2(a.s.k * f.x, 0.0) : make_double2(-a.s.k * f.y, a.s.k * f.x));
+    }
+    // rows nearer than this reach the lane's own damped by less than 2^-26
+    const double r = std::hypot(a.s.rinf.x, a.s.rinf.y);
+    a.near = 1;
+    for (double q = r; q >= 0x1p-26; q *= r) ++a.near;
+    return a;
+}
+
 template <int MODE, bool NL, bool P3> cudaError_t go_x(const SplitPlan &p, const IncArgs &a, cudaStream_t st)
 {
     auto kern = p.threads <= 256 ? k_inc_x<MODE, NL, P3, 256> : k_inc_x<MODE, NL, P3, kSplitThreads>;
@@ -717,6 +854,32 @@ cudaError_t go_yz(const SplitPlan &p, const IncArgs &a, cudaStream_t st)
 }
 
 }  // namespace
+
+cudaError_t launch_sweep_ffinc(const SplitPlan &p, int mode, void *psi, const AxisTables &ax, const SweepGeom &g,
+                               const FfNonlin *nl, const Partials *norm_out, cudaStream_t st)
+{
+    if (p.x ? norm_out != nullptr : nl != nullptr) return cudaErrorInvalidValue;
+    FfIncArgs a{};
+    a.i = inc_args(p, mode, psi, ax, g, nullptr, norm_out);
+    if (nl) {
+        a.px = nl->px;
+        a.i.s.py = nl->py;
+        a.i.s.pz = nl->pz;
+        a.i.s.sg = nl->g;
+        a.i.s.scale = nl->scale;
+    }
+    const bool small = p.threads <= 256;
+    void (*kern)(const FfIncArgs);
+#define GP_PICK(K, M, B) (small ? K<M, B, 256> : K<M, B, kSplitThreads>)
+    if (p.x && mode == 0) kern = nl ? GP_PICK(k_ffinc_x, 0, true) : GP_PICK(k_ffinc_x, 0, false);
+    else if (p.x) kern = nl ? GP_PICK(k_ffinc_x, 1, true) : GP_PICK(k_ffinc_x, 1, false);
+    else if (mode == 0) kern = norm_out ? GP_PICK(k_ffinc_yz, 0, true) : GP_PICK(k_ffinc_yz, 0, false);
+    else kern = norm_out ? GP_PICK(k_ffinc_yz, 1, true) : GP_PICK(k_ffinc_yz, 1, false);
+#undef GP_PICK
+    cudaError_t e = allow_smem(kern, p.smem);
+    if (e != cudaSuccess) return e;
+    return launch_after(p.after, kern, dim3(p.grid_x, p.grid_y), p.threads, p.smem, st, a);
+}
 
 bool rho_inc_plan(const RadialTables &rt, int nr, int nz, SplitPlan &p)
 {
@@ -775,17 +938,7 @@ size_t inc_extra_smem(int conv) { return inc_coef_bytes(conv); }
 cudaError_t launch_sweep_inc(const SplitPlan &p, int mode, void *psi, const AxisTables &ax, const SweepGeom &g,
                              const NonlinArgs *nl, bool nlout, const Partials *norm_out, cudaStream_t st)
 {
-    IncArgs a{};
-    a.s = split_args<kFp64>(p, mode, psi, ax, g, nl, norm_out);
-    a.rinf = ff_expand(a.s.rinf);
-    for (int q = 0; q < kIncEnds; ++q) {
-        const double2 f = a.s.mid[q];
-        a.kmid[q] = ff_expand(mode == 0 ? make_double2(a.s.k * f.x, 0.0) : make_double2(-a.s.k * f.y, a.s.k * f.x));
-    }
-    // rows nearer than this reach the lane's own damped by less than 2^-26
-    const double r = std::hypot(a.s.rinf.x, a.s.rinf.y);
-    a.near = 1;
-    for (double q = r; q >= 0x1p-26; q *= r) ++a.near;
+    const IncArgs a = inc_args(p, mode, psi, ax, g, nl, norm_out);
     const bool p3 = a.s.p3 != nullptr, norm = norm_out != nullptr;
     if (p.x) {
         if (nlout || norm || (p3 && mode == 0)) return cudaErrorInvalidValue;

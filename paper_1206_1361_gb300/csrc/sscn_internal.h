@@ -241,6 +241,10 @@ size_t inc_extra_smem(int conv);
 cudaError_t launch_sweep_inc(const SplitPlan &plan, int mode, void *psi, const AxisTables &ax,
                              const SweepGeom &g, const NonlinArgs *nl, bool nl_at_output,
                              const Partials *norm_out, cudaStream_t st);
+// The same on a float-float psi (plan: the complex128 one, plan.increment).  nl:
+// calcnu on every loaded point (x).
+cudaError_t launch_sweep_ffinc(const SplitPlan &plan, int mode, void *psi, const AxisTables &ax,
+                               const SweepGeom &g, const FfNonlin *nl, const Partials *norm_out, cudaStream_t st);
 // nl: calcnu on every loaded point (x), or with nl_at_output on every result
 // (real time, y / z); norm_out (imaginary time, y / z): as launch_sweep_yz.
 cudaError_t launch_sweep_split(const SplitPlan &plan, int prec, int mode, void *psi,

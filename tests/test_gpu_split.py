@@ -257,3 +257,20 @@ def test_axial_values_beyond_the_lifted_floats(scale):
     got = axial_run(nr, nz, 0.02, 0.0, gp.GP_REAL, psi0 * scale, 3) / scale
     # below the lifted range the increment is dropped: up to 8 kappa per sweep
     assert rel_l2(got, want) <= (1e-12 if scale > 1e-30 else 3 * 2 * 8 * 0.02)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("mode", [gp.GP_IMAG, gp.GP_REAL])
+@pytest.mark.parametrize("kappa", [0.006, 0.018])
+def test_float_float_matches_the_oracle(shape, mode, kappa):
+    """The float-float form on the sub-line sweeps: about 10 roundings of 2^-47 a
+    step, 3 steps: 2e-13 of the norm."""
+    require_gpu()
+    dt, g, steps, w = 1e-3, 4.0, 3, trap_of(shape)
+    h = spacing(shape, kappa, dt)
+    psi0 = rand_state(shape, 7)
+    got = run(shape, h, dt, w, g, mode, gp.GP_CFF, steps, psi0)
+    want = psi0.copy()
+    oracle.step(oracle_params(shape, h, dt, w, g, mode), want, steps)
+    assert rel_l2(got, want) <= 2e-13
