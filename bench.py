@@ -350,9 +350,10 @@ def autotune_entry(gp, ctx, case, precision, mode):
 
 def sweep_rooflines(gp, kt, points, precision, peaks, hbm_peak, hbm_src):
     """Roofline of the dominant sweep of a single-grid step from per-kernel
-    times: the arithmetic bound of its form (FP32 lane-operations for the
-    float-float form, FP64 flops for complex128; measured peaks) with the
-    HBM fraction of its algorithmic bytes beside it."""
+    times: the arithmetic bound of the float-float form (FP32 lane-operations;
+    measured peak) with the HBM fraction of its algorithmic bytes beside it;
+    for complex128, whose increments run on the FP32 pipe next to a few FP64
+    instructions a point, the HBM fraction."""
     sweeps = {k: v for k, v in kt.items() if k.startswith("sweep") and v > 0}
     dom = max(sweeps, key=sweeps.get)
     bpp = SWEEP_BYTES_PER_POINT[0]
@@ -364,10 +365,11 @@ def sweep_rooflines(gp, kt, points, precision, peaks, hbm_peak, hbm_src):
                     "%.1f T lane-operations/s)" % (peaks["fp32x2_fma"]["tflops"], peak))
         convention = "FP32 lane-operations (add, multiply or fused multiply-add on one lane = 1)"
     else:
-        ops = FLOPS_PER_POINT[gp.GP_REAL]
-        peak = peaks["fp64_fma"]["tflops"]
-        peak_src = "measured FP64 pipe rate (gp_measure_peak, DFMA)"
-        convention = "FP64 flops of the method's formulas"
+        return {"bound": "hbm", "kernel": dom, "achieved": hbm_achieved, "peak": hbm_peak,
+                "unit": "GB/s", "frac": hbm_achieved / hbm_peak, "peak_source": hbm_src,
+                "bytes_per_point": bpp,
+                "step_hbm_frac": (3 * bpp * points / 1e9) / (sum(sweeps.values()) * 1e-3) / hbm_peak,
+                "kernel_ms": {k: round(v, 5) for k, v in kt.items()}}
     achieved = ops[dom] * points / (sweeps[dom] * 1e-3) / 1e12
     return {"bound": "alu", "kernel": dom, "achieved": achieved, "peak": peak,
             "unit": "TFLOP/s", "frac": achieved / peak, "peak_source": peak_src,
@@ -541,9 +543,10 @@ def run_ours(args):
 
 
 def fp64_native_form(gp, torch, stream, case, ground, args, peaks, hbm_peak, hbm_src, ff_value):
-    """The same workload on the native FP64 form (complex128 psi, FP64 pipe):
-    the quench from the same ground state, the benchmark's step, its
-    throughput and the FP64-pipe roofline of its dominant sweep."""
+    """The same workload on the native FP64 form (complex128 psi, increments in
+    float-float arithmetic): the quench from the same ground state, the
+    benchmark's step, its throughput and the HBM fraction of its dominant
+    sweep."""
     ctx = gp.gp_create(case.shape, case.h, case.dt, *case.trap, case.g, gp.GP_REAL, gp.GP_C128,
                        stream)
     try:

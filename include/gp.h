@@ -294,7 +294,8 @@ enum {
      * truncation repeats identically every step, so it is kept far below
      * one rounding.  Under GP_PATH_AUTO a complex64 sweep reported as
      * GP_PATH_TMA runs its arithmetic on the cut lines where that is faster
-     * (small grids); a request for GP_PATH_TMA streams. */
+     * (small grids), and a float-float one the increment form on them; a
+     * request for GP_PATH_TMA streams. */
     GP_OPT_SWEEP_PATH = 1,
     /* Tile shape of the TMA sweep path: an index (0 .. GP_TILE_SHAPES - 1,
      * per precision) into the library's table of (lines per CTA, points per
