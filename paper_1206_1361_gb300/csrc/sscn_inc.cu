@@ -11,7 +11,7 @@
 // Here psi stays FP64, but the sweep computes the increment 2 Delta of
 //     (I - kappa L) Delta = kappa L psi,   u = psi + 2 Delta,
 // in float-float arithmetic (sscn_ff.cuh, ~48 significant bits) and adds it to
-// the FP64 psi: 2 FP64 instructions a point.  |2 Delta| is at most 8 kappa
+// the FP64 psi: 4 FP64 instructions a point (none with drop's MERGE).  |2 Delta| is at most 8 kappa
 // max|psi| and about kappa (k h)^2 |psi| on a smooth state, so with kappa up to
 // kIncKappaReal / kIncKappaImag the rounding of the increment stays at or below
 // that of the FP64 form u = 2 v - psi, which rounds at full size several times.
@@ -19,13 +19,14 @@
 // float-float, the potential factor multiplies in FP64.
 //
 // Measured (GB300, 256^3 real time, kappa = 0.0125): y and z sweeps 392 -> 226
-// us, x with calcnu 889 -> 432 us (8 FP64 instructions a point there: 230 us of
-// the FP64 pipe); the y sweep issues about 250 instructions a point, half of
-// them integer conversions and addresses, 56 % of the issue slots.  Relative L2
+// us, x with calcnu 889 -> 426 us (8 FP64 instructions a point there: 230 us of
+// the FP64 pipe); the y sweep issues about 320 instructions a point, half of
+// them integer conversions and addresses, 62 % of the issue slots, with the FP64
+// pipe 57 % busy (x: 540, 55 % and 53 %).  Relative L2
 // error against FP64 truth, start and here: 64^3 imaginary, 100 steps, 5.3e-15
 // and 2.1e-15; 256^3 real, 10 steps, 6.8e-15 and 4.4e-15; 128 x 96 x 80 real at
 // kappa = 0.05, 20 steps, 1.5e-14 and 6.6e-15.  In imaginary time the state
-// hardly changes from step to step and the rounding of the lifted psi repeats:
+// hardly changes from step to step and the rounding repeats:
 // at kappa = 0.05 (500 x 384, 40 steps) 2.4e-15 against 1.6e-15, hence the
 // smaller kIncKappaImag.  In real time the error moves with kappa through the
 // rounding of the coefficients, the same at every step, in both forms; over
