@@ -846,7 +846,7 @@ IncArgs inc_args(const SplitPlan &p, int mode, void *psi, const AxisTables &ax, 
 template <int MODE, bool NL, bool P3> cudaError_t go_x(const SplitPlan &p, const IncArgs &a, cudaStream_t st)
 {
     auto kern = p.threads <= 256 ? k_inc_x<MODE, NL, P3, 256> : k_inc_x<MODE, NL, P3, kSplitThreads>;
-    cudaError_t e = allow_smem(kern, p.smem);
+    cudaError_t e = allow_smem(kern);
     if (e != cudaSuccess) return e;
     return launch_after(p.after, kern, p.grid_x, p.threads, p.smem, st, a);
 }
@@ -855,7 +855,7 @@ template <int MODE, bool NORM, bool NLOUT, bool P3>
 cudaError_t go_yz(const SplitPlan &p, const IncArgs &a, cudaStream_t st)
 {
     auto kern = p.threads <= 256 ? k_inc_yz<MODE, NORM, NLOUT, P3, 256> : k_inc_yz<MODE, NORM, NLOUT, P3, kSplitThreads>;
-    cudaError_t e = allow_smem(kern, p.smem);
+    cudaError_t e = allow_smem(kern);
     if (e != cudaSuccess) return e;
     return launch_after(p.after, kern, dim3(p.grid_x, p.grid_y), p.threads, p.smem, st, a);
 }
@@ -883,7 +883,7 @@ cudaError_t launch_sweep_ffinc(const SplitPlan &p, int mode, void *psi, const Ax
     else if (mode == 0) kern = norm_out ? GP_PICK(k_ffinc_yz, 0, true) : GP_PICK(k_ffinc_yz, 0, false);
     else kern = norm_out ? GP_PICK(k_ffinc_yz, 1, true) : GP_PICK(k_ffinc_yz, 1, false);
 #undef GP_PICK
-    cudaError_t e = allow_smem(kern, p.smem);
+    cudaError_t e = allow_smem(kern);
     if (e != cudaSuccess) return e;
     return launch_after(p.after, kern, dim3(p.grid_x, p.grid_y), p.threads, p.smem, st, a);
 }
@@ -933,7 +933,7 @@ cudaError_t launch_sweep_rho_inc(const SplitPlan &p, int mode, void *psi, void *
     a.rt = rt;
     auto kern = p.threads <= 256 ? (mode == 0 ? k_inc_rho<0, 256> : k_inc_rho<1, 256>)
                                  : (mode == 0 ? k_inc_rho<0, kSplitThreads> : k_inc_rho<1, kSplitThreads>);
-    cudaError_t e = allow_smem(kern, p.smem);
+    cudaError_t e = allow_smem(kern);
     if (e != cudaSuccess) return e;
     return launch_after(p.after, kern, p.grid_x, p.threads, p.smem, st, a);
 }

@@ -353,7 +353,7 @@ template <int FORM, int MODE, bool NL, bool P3, int P, typename T>
 cudaError_t go_x(const SplitPlan &p, const SplitArgs<T> &a, cudaStream_t st)
 {
     auto kern = k_split_x<FORM, MODE, NL, P3, P>;
-    cudaError_t e = allow_smem(kern, p.smem);
+    cudaError_t e = allow_smem(kern);
     if (e != cudaSuccess) return e;
     return launch_after(p.after, kern, p.grid_x, p.threads, p.smem, st, a);
 }
@@ -362,7 +362,7 @@ template <int FORM, int MODE, bool NORM, bool NLOUT, bool P3, int P, typename T>
 cudaError_t go_yz(const SplitPlan &p, const SplitArgs<T> &a, cudaStream_t st)
 {
     auto kern = k_split_yz<FORM, MODE, NORM, NLOUT, P3, P>;
-    cudaError_t e = allow_smem(kern, p.smem);
+    cudaError_t e = allow_smem(kern);
     if (e != cudaSuccess) return e;
     return launch_after(p.after, kern, dim3(p.grid_x, p.grid_y), p.threads, p.smem, st, a);
 }

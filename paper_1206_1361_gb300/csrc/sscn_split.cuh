@@ -246,12 +246,15 @@ __device__ __forceinline__ void block_partial(double part, double *red, double *
     }
 }
 
-// All of an SM's shared memory for resident blocks, and as much as a block needs.
-template <typename K> cudaError_t allow_smem(K kern, size_t bytes)
+// All of an SM's shared memory for resident blocks, and as much as any block of
+// these kernels needs: without this a block's static and dynamic shared memory
+// together may not pass 48 KB, so the dynamic part alone does not say whether
+// it is needed.
+template <typename K> cudaError_t allow_smem(K kern)
 {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
                                          (int)cudaSharedmemCarveoutMaxShared);
-    if (e != cudaSuccess || bytes <= 48 * 1024) return e;
+    if (e != cudaSuccess) return e;
     return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSplitSmem);
 }
 
