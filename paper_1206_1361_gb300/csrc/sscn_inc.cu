@@ -76,50 +76,51 @@ struct IncArgs {
 
 // ------------------------------------------------------------- conversions
 
-constexpr unsigned kOff = (unsigned)(1023 - 127 - kLift) << 20;   // FP64 - FP32 exponent, lifted
+// FP64 - FP32 exponent in the high word, of values multiplied by 2^e on the way.
+__host__ __device__ constexpr unsigned offset_of(int e) { return (unsigned)(1023 - 127 - e) << 20; }
+constexpr unsigned kOff = offset_of(kLift);
 
 // Not finite, or too large for a lifted float (MARGIN: times 2^MARGIN).
-template <int MARGIN = 0> __device__ __forceinline__ bool too_large(double x)
+template <int MARGIN = 0> __device__ __forceinline__ bool too_large(double x, unsigned off = kOff)
 {
-    return ((unsigned)__double2hiint(x) & 0x7fffffffu) >= kOff + ((250u - MARGIN) << 20);
+    return ((unsigned)__double2hiint(x) & 0x7fffffffu) >= off + ((250u - MARGIN) << 20);
 }
 
-// 2^kLift x as a float-float pair: hi the nearest float (ties away from zero),
+// 2^e x (off: offset_of(e)) as a float-float pair: hi the nearest float (ties away from zero),
 // lo the float nearest the rest.  With x = s m 2^(e-52), m the 53-bit
 // significand: hi = s r 2^(e-23), r = (m + 2^28) >> 29, and x - hi = s d
 // 2^(e-52), d = m - 2^29 r = ((m + 2^28) mod 2^29) - 2^28.
-__device__ __forceinline__ float2 lift(double x)
+__device__ __forceinline__ float2 lift(double x, unsigned off)
 {
     const unsigned L = (unsigned)__double2loint(x), H = (unsigned)__double2hiint(x);
-    const unsigned L2 = L + 0x10000000u, E = H - kOff, E2 = E + (L2 < L ? 1u : 0u);
-    const unsigned sign = H & 0x80000000u, mag = H & 0x7fffffffu;
-    float hi = __uint_as_float((__funnelshift_l(L2, E2, 3) & 0x7fffffffu) | sign);
+    const unsigned sign = H & 0x80000000u, L2 = L + 0x10000000u;
+    const int E = (int)((H & 0x7fffffffu) - off), E2 = E + (L2 < L ? 1 : 0);
+    float hi = __uint_as_float(__funnelshift_l(L2, (unsigned)E2, 3) | sign);
     const int d = (int)(L2 & 0x1fffffffu) - 0x10000000;
-    const float ulp = __uint_as_float((((E - (52u << 20)) << 3) & 0x7f800000u) | sign);   // s 2^(e-52)
+    const float ulp = __uint_as_float((((unsigned)(E - (52 << 20)) << 3) & 0x7f800000u) | sign);   // s 2^(e-52)
     float lo = __int2float_rn(d) * ulp;
-    if (mag < kOff + (53u << 20)) lo = 0.f;
-    if (mag < kOff + (1u << 20)) hi = 0.f;
+    if (E < (53 << 20)) lo = 0.f;
+    if (E < (1 << 20)) hi = 0.f;
     return f2(hi, lo);
 }
 
-// 2^TIMES x (SCALED: x lifted) as FP64: exact, zero for zero.
-template <int TIMES, bool SCALED> __device__ __forceinline__ double widen(float x)
+// 2^-e x (off: offset_of(e)) as FP64: exact, zero for zero.
+__device__ __forceinline__ double widen(float x, unsigned off)
 {
-    constexpr unsigned off = (SCALED ? kOff : (unsigned)(1023 - 127) << 20) + ((unsigned)TIMES << 20);
     const unsigned f = __float_as_uint(x), mag = f & 0x7fffffffu;
     const unsigned H = mag == 0u ? 0u : (mag >> 3) + off;
     return __hiloint2double((int)(H | (f & 0x80000000u)), (int)(f << 29));
 }
 
-// 2^(TIMES - kLift) (hi + lo) as FP64 with one FP64 addition; or (MERGE) with
+// 2^-e (hi + lo) as FP64 with one FP64 addition; or (MERGE) with
 // none: hi's bits as FP64 bits plus lo, renormalised to at most half an ulp of
 // hi, in units of FP64's last place (carries and borrows run through the
 // exponent field as they should; below a power of two the place is half as
 // large).  MERGE takes about 12 more instructions: for the x sweep, which the
 // FP64 pipe bounds.
-template <int TIMES, bool SCALED, bool MERGE> __device__ __forceinline__ double drop(float h, float l)
+template <bool MERGE> __device__ __forceinline__ double drop(float h, float l, unsigned off)
 {
-    if (!MERGE) return widen<TIMES, SCALED>(h) + widen<TIMES, SCALED>(l);
+    if (!MERGE) return widen(h, off) + widen(l, off);
     const float2 z = ff::s_two_sum(h, l);
     const unsigned f = __float_as_uint(z.x), ef = f & 0x7f800000u;
     const float units = __uint_as_float(ef >= (53u << 23) ? (306u << 23) - ef : 0u);      // 2^(52 - e)
@@ -127,21 +128,21 @@ template <int TIMES, bool SCALED, bool MERGE> __device__ __forceinline__ double 
     const int neg = (int)f >> 31;
     li = (li ^ neg) - neg;
     if ((f & 0x7fffffu) == 0u && li < 0) li *= 2;
-    const long long b = __double_as_longlong(widen<TIMES, SCALED>(z.x)) + (long long)li;
+    const long long b = __double_as_longlong(widen(z.x, off)) + (long long)li;
     return ef == 0u ? 0.0 : __longlong_as_double(b);
 }
 
-__device__ __forceinline__ FC lift(double2 p)
+__device__ __forceinline__ FC lift(double2 p, unsigned off = kOff)
 {
-    const float2 x = lift(p.x), y = lift(p.y);
+    const float2 x = lift(p.x, off), y = lift(p.y, off);
     return FC{f2(x.x, y.x), f2(x.y, y.y)};
 }
 
-// p + 2^(TIMES - kLift) z
-template <int TIMES, bool MERGE> __device__ __forceinline__ double2 plus(double2 p, FC z)
+// p + 2^TIMES z, z lifted
+template <int TIMES, bool MERGE> __device__ __forceinline__ double2 plus(double2 p, FC z, unsigned off = kOff)
 {
-    return make_double2(p.x + drop<TIMES, true, MERGE>(z.hi.x, z.lo.x),
-                        p.y + drop<TIMES, true, MERGE>(z.hi.y, z.lo.y));
+    off += (unsigned)TIMES << 20;
+    return make_double2(p.x + drop<MERGE>(z.hi.x, z.lo.x, off), p.y + drop<MERGE>(z.hi.y, z.lo.y, off));
 }
 
 __device__ __forceinline__ float4 pack(FC z) { return make_float4(z.hi.x, z.hi.y, z.lo.x, z.lo.y); }
@@ -149,61 +150,74 @@ __device__ __forceinline__ FC unpack(float4 v) { return FC{f2(v.x, v.y), f2(v.z,
 
 // ------------------------------------------------------------------ calcnu
 
-// G 2^(-2 kLift) as a pair: times |lift(p)|^2 it gives a = G |p|^2.
-__device__ __forceinline__ float2 lifted_g(double G)
+// G of the step, and G 2^(-2 k) as a pair with the offset of values times 2^k: a =
+// G |p|^2 is formed as (G 2^(-2 k)) |2^k p|^2 with k from G's exponent, so that
+// where the series below serves (|a| < 2^-8) |2^k p| is below 2^-3 whatever the
+// units of psi and G, and what underflows belongs to an a below 2^-90.  (With
+// psi's own lift, G of a |psi| beyond 10^6 fell among the denormals.)
+struct NlScale {
+    double G;
+    float2 g;
+    unsigned off;
+};
+
+__device__ __forceinline__ NlScale nl_scale(double G)
 {
-    const double g = ldexp(G, -2 * kLift);
+    const int e = (__double2hiint(G) >> 20) & 0x7ff;
+    // 2^(-2 k) G in [1/2, 2); zero and what is not finite as they are
+    const int k = e == 0 ? (G == 0.0 ? 0 : -512) : e == 0x7ff ? 0 : (e - 1022) >> 1;
+    const double s = __hiloint2double((1023 - k) << 20, 0), g = G * s * s;
     const float h = (float)g;
-    return f2(h, (float)(g - (double)h));
+    return NlScale{G, f2(h, (float)(g - (double)h)), offset_of(k)};
 }
 
 // Real time: exp(-i a) p, a = G |p|^2, as p + (exp(-i a) - 1) p with the factor
 // from its Taylor series in float-float for |a| < 2^-8 (first dropped terms
 // a^6 / 720 and a^7 / 5040 below 2^-57), in FP64 beyond.
-__device__ __forceinline__ double2 nonlinear_real(double2 p, float2 g, double G)
+__device__ __forceinline__ double2 nonlinear_real(double2 p, const NlScale &s)
 {
-    const FC z = lift(p);
-    const float2 a = ff::s_mul(g, ff::abs2(z));
-    if (fabsf(a.x) < 0x1p-8f && !too_large(p.x) && !too_large(p.y)) {
+    const FC z = lift(p, s.off);
+    const float2 a = ff::s_mul(s.g, ff::abs2(z));
+    if (fabsf(a.x) < 0x1p-8f && !too_large(p.x, s.off) && !too_large(p.y, s.off)) {
         const float q = __fmul_rn(a.x, a.x);
         float qe = fmaf(a.x, a.x, -q);
         qe = fmaf(2.f * a.x, a.y, qe);
         const float2 dr = f2(-0.5f * q, fmaf(q * q, 1.f / 24, -0.5f * qe));
         const float2 di = f2(-a.x, fmaf(a.x * q, fmaf(q, -1.f / 120, 1.f / 6), -a.y));
         const FfCoef D{f2(dr.x, dr.x), f2(dr.y, dr.y), f2(-di.x, di.x), f2(-di.y, di.y)};
-        return plus<0, true>(p, ff::cmul(z, D));
+        return plus<0, true>(p, ff::cmul(z, D), s.off);
     }
     double cs, sn;
-    expmi_small(G * fma(p.x, p.x, p.y * p.y), cs, sn);
+    expmi_small(s.G * fma(p.x, p.x, p.y * p.y), cs, sn);
     return make_double2(fma(cs, p.x, sn * p.y), fma(cs, p.y, -sn * p.x));
 }
 
 // Imaginary time: f exp(-a), a = G |p|^2, as f + f (exp(-a) - 1) likewise.
-__device__ __forceinline__ double factor_imag(double2 p, double f, float2 g, double G)
+__device__ __forceinline__ double factor_imag(double2 p, double f, const NlScale &s)
 {
-    const float2 a = ff::s_mul(g, ff::abs2(lift(p)));
-    if (fabsf(a.x) < 0x1p-8f && !too_large(p.x) && !too_large(p.y)) {
+    const float2 a = ff::s_mul(s.g, ff::abs2(lift(p, s.off)));
+    if (fabsf(a.x) < 0x1p-8f && !too_large(p.x, s.off) && !too_large(p.y, s.off)) {
         const float q = __fmul_rn(a.x, a.x);
         float qe = fmaf(a.x, a.x, -q);
         qe = fmaf(2.f * a.x, a.y, qe);
-        const float2 s = ff::s_two_sum(-a.x, 0.5f * q);
+        const float2 d = ff::s_two_sum(-a.x, 0.5f * q);
         const float tail = fmaf(q, fmaf(a.x, -1.f / 120, 1.f / 24) * q, -a.x * q * (1.f / 6));
-        const float2 eps = ff::s_norm(f2(s.x, s.y + ((0.5f * qe - a.y) + tail)));
-        return fma(f, drop<0, false, true>(eps.x, eps.y), f);
+        const float2 eps = ff::s_norm(f2(d.x, d.y + ((0.5f * qe - a.y) + tail)));
+        return fma(f, drop<true>(eps.x, eps.y, offset_of(0)), f);
     }
-    return f * expm_small(G * fma(p.x, p.x, p.y * p.y));
+    return f * expm_small(s.G * fma(p.x, p.x, p.y * p.y));
 }
 
 // calcnu at stored point i (MODE 0: c.pyz carries the pending scale).
 template <int MODE, bool P3>
-__device__ __forceinline__ double2 calcnu_at(double2 p, const Calcnu<double, MODE> &c, int i, double2 p3, float2 g,
-                                             double G)
+__device__ __forceinline__ double2 calcnu_at(double2 p, const Calcnu<double, MODE> &c, int i, double2 p3,
+                                             const NlScale &s)
 {
     if (MODE == 0) {
-        const double f = factor_imag(p, c.pyz.x * c.px[i].x, g, G);
+        const double f = factor_imag(p, c.pyz.x * c.px[i].x, s);
         return make_double2(p.x * f, p.y * f);
     }
-    const double2 w = nonlinear_real(p, g, G);
+    const double2 w = nonlinear_real(p, s);
     return P3 ? cmulc(w, p3) : cmulc(cmulc(w, c.pyz), c.px[i]);
 }
 
@@ -455,8 +469,7 @@ template <int MODE, bool NL, bool P3, int THREADS>
 __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_x(const __grid_constant__ IncArgs A)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ double g_of_step;
-    __shared__ float2 g_lifted;
+    __shared__ NlScale nl_of_step;
     const SplitArgs<double> &a = A.s;
     const int n = a.n, pitch = slot_of(n) + 1;
     unsigned char *coef = smem_raw, *coef64 = coef + inc_coef_bytes(a.conv);
@@ -487,8 +500,7 @@ __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_x(const __
     }
     if (NL && threadIdx.x == 0) {
         const double G = a.sg.value(), sc = MODE == 0 && a.scale ? *a.scale : 1.0;
-        g_of_step = G * sc * sc;
-        g_lifted = lifted_g(G * sc * sc);
+        nl_of_step = nl_scale(G * sc * sc);
     }
     if (NL && !P3)
         for (int r = threadIdx.x; r < rows; r += blockDim.x) {
@@ -498,14 +510,13 @@ __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_x(const __
     if (NL) __syncthreads();                 // row_nl, G
     bool big = false;
     if (active) {
-        const double G = NL ? g_of_step : 0.0;
-        const float2 gl = NL ? g_lifted : f2(0.f, 0.f);
+        const NlScale ns = NL ? nl_of_step : NlScale{};
 #pragma unroll
         for (int b = 0; b < kIncP; ++b) {
             const int i = 1 + seg + b * lanes;
             if (i < n) {
                 if constexpr (NL) {
-                    v[b] = calcnu_at<MODE, P3>(v[b], row_nl[P3 ? 0 : q], i, f3[P3 ? b : 0], gl, G);
+                    v[b] = calcnu_at<MODE, P3>(v[b], row_nl[P3 ? 0 : q], i, f3[P3 ? b : 0], ns);
                     row[i] = v[b];
                 }
                 big = big || too_large(v[b].x) || too_large(v[b].y);
@@ -549,8 +560,8 @@ template <int MODE, bool NORM, bool NLOUT, bool P3, int THREADS>
 __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_yz(const __grid_constant__ IncArgs A)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ double red[32], g_of_step;
-    __shared__ float2 g_lifted;
+    __shared__ double red[32];
+    __shared__ NlScale nl_of_step;
     const SplitArgs<double> &a = A.s;
     unsigned char *coef = smem_raw, *coef64 = coef + inc_coef_bytes(a.conv);
     float4 *tile = reinterpret_cast<float4 *>(coef64 + coef_bytes<double>(a.conv));
@@ -563,10 +574,7 @@ __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_yz(const _
     double2 *line = a.psi + base;
     stage_inc<MODE>(A, coef);
     pdl_wait();
-    if (NLOUT && threadIdx.x == 0) {
-        g_of_step = a.sg.value();
-        g_lifted = lifted_g(g_of_step);
-    }
+    if (NLOUT && threadIdx.x == 0) nl_of_step = nl_scale(a.sg.value());
     auto at_of = [&](int i) { return slot_of(i) * XL + xl; };
     bool big = false;
     if (active) {
@@ -585,8 +593,7 @@ __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_yz(const _
     }
     big = __syncthreads_or(big);
     Calcnu<double, MODE> nl{};
-    const double G = NLOUT ? g_of_step : 0.0;
-    const float2 gl = NLOUT ? g_lifted : f2(0.f, 0.f);
+    const NlScale ns = NLOUT ? nl_of_step : NlScale{};
     if (NLOUT && !P3 && active) nl.setup(a.px, a.py, a.pz, nullptr, nullptr, nullptr, la, lb, 0.0, nullptr);
     double acc = 0.0;
     auto finish = [&](int i, double2 u) {
@@ -594,7 +601,7 @@ __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_yz(const _
         if constexpr (NLOUT) {
             double2 f = make_double2(0.0, 0.0);
             if constexpr (P3) f = a.p3[base + at];
-            u = calcnu_at<MODE, P3>(u, nl, i, f, gl, G);
+            u = calcnu_at<MODE, P3>(u, nl, i, f, ns);
         }
         line[at] = u;
         if (NORM) acc = fma(u.x, u.x, fma(u.y, u.y, acc));
@@ -755,8 +762,7 @@ template <int MODE, int THREADS>
 __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_rho(const __grid_constant__ RadArgs A)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ double g_of_step;
-    __shared__ float2 g_lifted;
+    __shared__ NlScale nl_of_step;
     const SplitArgs<double> &a = A.s;
     const int n = a.n, m = n - 1, pitch = slot_of(n) + 1;
     float4 *coef = reinterpret_cast<float4 *>(smem_raw);
@@ -786,21 +792,19 @@ __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_rho(const 
     }
     if (threadIdx.x == 0) {
         const double G = a.sg.value(), sc = MODE == 0 && a.scale ? *a.scale : 1.0;
-        g_of_step = G * sc * sc;
-        g_lifted = lifted_g(G * sc * sc);
+        nl_of_step = nl_scale(G * sc * sc);
     }
     for (int r = threadIdx.x; r < rows; r += blockDim.x)
         row_nl[r].setup(a.px, a.py, a.pz, nullptr, nullptr, nullptr, line0 + r, 0, 0.0, a.scale);
     __syncthreads();                         // row_nl, G
     bool big = false;
     if (active) {
-        const double G = g_of_step;
-        const float2 gl = g_lifted;
+        const NlScale ns = nl_of_step;
 #pragma unroll
         for (int b = 0; b < kIncP; ++b) {
             const int i = seg + b * lanes;
             if (i < m) {
-                v[b] = calcnu_at<MODE, false>(v[b], row_nl[q], i, make_double2(0.0, 0.0), gl, G);
+                v[b] = calcnu_at<MODE, false>(v[b], row_nl[q], i, make_double2(0.0, 0.0), ns);
                 row[i] = v[b];
                 big = big || too_large<kRadialBits>(v[b].x) || too_large<kRadialBits>(v[b].y);
                 tile[at + slot_of(i + 1)] = pack(lift(v[b]));
