@@ -69,8 +69,10 @@ enum { GP_IMAG = 0, GP_REAL = 1 };           /* propagation mode            */
  * psi / sweep precision.  GP_C128: complex128 psi, FP64 arithmetic; where
  * kappa = dt / (4 h^2) is small (<= 0.025 in imaginary, 0.06 in real time) the
  * default path adds to the FP64 psi an increment computed in float-float
- * arithmetic, with a smaller rounding error than FP64 sweeps (amplitudes
- * below 2^-105 carry theirs to 24 bits).
+ * arithmetic, with a smaller rounding error than FP64 sweeps.  Relative to
+ * the largest amplitude of the lines that a block sweeps together, one 2^-30
+ * times as large or smaller may carry its increment to 24 bits, one 2^-81
+ * times as large or smaller none.
  * GP_C64: complex64 psi and sweeps, FP64 tables and reductions.
  * GP_CFF: the FP64-class float-float form -- psi is kept on the device as
  * float-float pairs (per point four floats: re_hi, im_hi, re_lo, im_lo,

@@ -48,7 +48,12 @@
 // Conversions go through the bits of the double with integer instructions (the
 // FP64 <-> FP32 conversion instructions run on the FP64 pipe).  Values enter
 // multiplied by 2^kLift, which puts the full float-float precision at 2^-105
-// .. 2^93; a block that holds anything larger, or not finite, sweeps in FP64.
+// .. 2^93.  A block whose largest value lies below 2^-75 (psi is small
+// everywhere, or its lines run far outside the cloud) or above 2^93 lifts it to
+// 2^20 instead; outside 2^-800 .. 2^1000, and with anything not finite, it
+// sweeps in FP64.  So an increment that comes with fewer bits (values below
+// 2^-105) or none (below 2^-156) belongs to a value 2^30 or 2^81 times smaller
+// than the block's largest.
 
 #include "sscn_ff.cuh"
 #include "sscn_rho.cuh"
@@ -80,10 +85,13 @@ struct IncArgs {
 __host__ __device__ constexpr unsigned offset_of(int e) { return (unsigned)(1023 - 127 - e) << 20; }
 constexpr unsigned kOff = offset_of(kLift);
 
-// Not finite, or too large for a lifted float (MARGIN: times 2^MARGIN).
-template <int MARGIN = 0> __device__ __forceinline__ bool too_large(double x, unsigned off = kOff)
+// High word from which on a value is too large for a float lifted with off, or not
+// finite (with 2^margin to spare).
+__host__ __device__ constexpr unsigned most_of(unsigned off, unsigned margin = 0) { return off + ((250u - margin) << 20); }
+
+__device__ __forceinline__ bool too_large(double x, unsigned off)
 {
-    return ((unsigned)__double2hiint(x) & 0x7fffffffu) >= off + ((250u - MARGIN) << 20);
+    return ((unsigned)__double2hiint(x) & 0x7fffffffu) >= most_of(off);
 }
 
 // 2^e x (off: offset_of(e)) as a float-float pair: hi the nearest float (ties away from zero),
@@ -104,11 +112,11 @@ __device__ __forceinline__ float2 lift(double x, unsigned off)
     return f2(hi, lo);
 }
 
-// 2^-e x (off: offset_of(e)) as FP64: exact, zero for zero.
+// 2^-e x (off: offset_of(e)) as FP64: exact, zero for zero and FP32 denormals.
 __device__ __forceinline__ double widen(float x, unsigned off)
 {
     const unsigned f = __float_as_uint(x), mag = f & 0x7fffffffu;
-    const unsigned H = mag == 0u ? 0u : (mag >> 3) + off;
+    const unsigned H = mag < 0x800000u ? 0u : (mag >> 3) + off;
     return __hiloint2double((int)(H | (f & 0x80000000u)), (int)(f << 29));
 }
 
@@ -147,6 +155,39 @@ template <int TIMES, bool MERGE> __device__ __forceinline__ double2 plus(double2
 
 __device__ __forceinline__ float4 pack(FC z) { return make_float4(z.hi.x, z.hi.y, z.lo.x, z.lo.y); }
 __device__ __forceinline__ FC unpack(float4 v) { return FC{f2(v.x, v.y), f2(v.z, v.w)}; }
+
+// The largest magnitude a lane has seen, as a high word; 1 for an FP64 denormal
+// whose high word is zero.
+struct Seen {
+    unsigned top = 0, low = 0;
+
+    __device__ __forceinline__ void add(double2 p)
+    {
+        top = max(top, max((unsigned)__double2hiint(p.x) & 0x7fffffffu, (unsigned)__double2hiint(p.y) & 0x7fffffffu));
+        low |= (unsigned)__double2loint(p.x) | (unsigned)__double2loint(p.y);
+    }
+    __device__ __forceinline__ unsigned value() const { return top == 0u && low != 0u ? 1u : top; }
+};
+
+// The offset of the block's lift, from what its lanes have seen; 0: the block
+// sweeps in FP64.  One barrier where
+// every lane has seen ordinary values or zeros only, three more otherwise.
+template <int MARGIN = 0> __device__ __forceinline__ unsigned block_offset(const Seen &seen)
+{
+    constexpr unsigned most = most_of(kOff, MARGIN), tiny = (1023u - 75u) << 20;
+    constexpr unsigned least = (1023u - 800u) << 20, huge = (1023u + 1000u) << 20;
+    __shared__ unsigned block_top;
+    unsigned top = seen.value();
+    if (!__syncthreads_or(top != 0u && top - tiny >= most - tiny)) return kOff;
+    if (threadIdx.x == 0) block_top = 0u;
+    __syncthreads();
+    top = __reduce_max_sync(0xffffffffu, top);
+    if ((threadIdx.x & 31) == 0) atomicMax(&block_top, top);
+    __syncthreads();
+    top = block_top;
+    if (top >= tiny && top < most) return kOff;
+    return top >= least && top < huge ? ((top >> 20) - 127u - 20u) << 20 : 0u;
+}
 
 // ------------------------------------------------------------------ calcnu
 
@@ -508,7 +549,7 @@ __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_x(const __
             row_nl[r].setup(a.px, a.py, a.pz, nullptr, nullptr, nullptr, L % a.lines_a, L / a.lines_a, 0.0, a.scale);
         }
     if (NL) __syncthreads();                 // row_nl, G
-    bool big = false;
+    Seen seen;
     if (active) {
         const NlScale ns = NL ? nl_of_step : NlScale{};
 #pragma unroll
@@ -519,13 +560,14 @@ __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_x(const __
                     v[b] = calcnu_at<MODE, P3>(v[b], row_nl[P3 ? 0 : q], i, f3[P3 ? b : 0], ns);
                     row[i] = v[b];
                 }
-                big = big || too_large(v[b].x) || too_large(v[b].y);
+                seen.add(v[b]);
                 tile[at + slot_of(i)] = pack(lift(v[b]));
             }
         }
     }
     const int own = active ? seg : (threadIdx.x & 1);
-    if (__syncthreads_or(big)) {
+    const unsigned off = block_offset(seen);
+    if (off == 0u) {
         double2 *t64 = reinterpret_cast<double2 *>(tile);
         stage_coefs<MODE>(a, coef64);
         if (active)
@@ -540,6 +582,11 @@ __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_x(const __
             for (int i = 1 + seg; i < n; i += lanes) row[i] = t64[at + slot_of(i)];
         return;
     }
+    if (off != kOff) {
+        if (active)
+            for (int i = 1 + seg; i < n; i += lanes) tile[at + slot_of(i)] = pack(lift(row[i], off));
+        __syncthreads();
+    }
     const IncLane<MODE> lane(A, coef, own);
     lane.template solve<true>(
         active, 1, [&](int i) { return unpack(tile[at + slot_of(i)]); },
@@ -549,19 +596,23 @@ __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_x(const __
 #pragma unroll
         for (int b = 0; b < kIncP; ++b) {
             const int i = 1 + seg + b * lanes;
-            if (i < n) row[i] = plus<1, true>(row[i], unpack(tile[at + slot_of(i)]));
+            if (i < n) row[i] = plus<1, true>(row[i], unpack(tile[at + slot_of(i)]), off);
         }
     }
 }
 
 // y / z sweep: as k_split_yz; a lane reads the FP64 values of its rows again
-// (from L1 or L2) when it adds the increments.
+// (from L1 or L2) when it adds the increments.  Without calcnu the lift's offset
+// waits in shared memory: a register for it spilled (256^3 real time 880 us a
+// step with it, 876 so, 872 with a constant lift).
 template <int MODE, bool NORM, bool NLOUT, bool P3, int THREADS>
 __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_yz(const __grid_constant__ IncArgs A)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double red[32];
     __shared__ NlScale nl_of_step;
+    __shared__ volatile unsigned lift_off;
+    if (threadIdx.x == 0) lift_off = kOff;
     const SplitArgs<double> &a = A.s;
     unsigned char *coef = smem_raw, *coef64 = coef + inc_coef_bytes(a.conv);
     float4 *tile = reinterpret_cast<float4 *>(coef64 + coef_bytes<double>(a.conv));
@@ -576,7 +627,7 @@ __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_yz(const _
     pdl_wait();
     if (NLOUT && threadIdx.x == 0) nl_of_step = nl_scale(a.sg.value());
     auto at_of = [&](int i) { return slot_of(i) * XL + xl; };
-    bool big = false;
+    Seen seen;
     if (active) {
         double2 p[kIncP];
 #pragma unroll
@@ -585,13 +636,13 @@ __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_yz(const _
 #pragma unroll
         for (int q = 0; q < kIncP; ++q)
             if (lane.first + q <= lane.last) {
-                big = big || too_large(p[q].x) || too_large(p[q].y);
+                seen.add(p[q]);
                 tile[at_of(lane.row(lane.first + q))] = pack(lift(p[q]));
             }
         if (seg == 0) tile[at_of(0)] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (seg == 1) tile[at_of(n)] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    big = __syncthreads_or(big);
+    const unsigned off = block_offset(seen);
     Calcnu<double, MODE> nl{};
     const NlScale ns = NLOUT ? nl_of_step : NlScale{};
     if (NLOUT && !P3 && active) nl.setup(a.px, a.py, a.pz, nullptr, nullptr, nullptr, la, lb, 0.0, nullptr);
@@ -606,7 +657,7 @@ __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_yz(const _
         line[at] = u;
         if (NORM) acc = fma(u.x, u.x, fma(u.y, u.y, acc));
     };
-    if (big) {
+    if (off == 0u) {
         double2 *t64 = reinterpret_cast<double2 *>(tile);
         stage_coefs<MODE>(a, coef64);
         if (active) {
@@ -622,9 +673,21 @@ __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_yz(const _
         lane64.template solve<kIncP, false>(
             active, XL, [&](int i) { return t64[at_of(i)]; }, 0, 0, finish);
     } else {
+        if (off != kOff) {
+            if (threadIdx.x == 0) lift_off = off;
+            if (active) {
+#pragma unroll
+                for (int q = 0; q < kIncP; ++q)
+                    if (lane.first + q <= lane.last) {
+                        const int i = lane.row(lane.first + q);
+                        tile[at_of(i)] = pack(lift(line[(long long)i * a.pstride], off));
+                    }
+            }
+            __syncthreads();
+        }
         lane.template solve<false>(
             active, XL, [&](int i) { return unpack(tile[at_of(i)]); },
-            [&](int, int i, FC g) { finish(i, plus<1, false>(line[(long long)i * a.pstride], g)); });
+            [&](int, int i, FC g) { finish(i, plus<1, false>(line[(long long)i * a.pstride], g, NLOUT ? off : lift_off)); });
     }
     if (NORM) {
         if (a.lw && active) acc *= a.lw[la];
@@ -797,7 +860,7 @@ __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_rho(const 
     for (int r = threadIdx.x; r < rows; r += blockDim.x)
         row_nl[r].setup(a.px, a.py, a.pz, nullptr, nullptr, nullptr, line0 + r, 0, 0.0, a.scale);
     __syncthreads();                         // row_nl, G
-    bool big = false;
+    Seen seen;
     if (active) {
         const NlScale ns = nl_of_step;
 #pragma unroll
@@ -806,16 +869,22 @@ __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_rho(const 
             if (i < m) {
                 v[b] = calcnu_at<MODE, false>(v[b], row_nl[q], i, make_double2(0.0, 0.0), ns);
                 row[i] = v[b];
-                big = big || too_large<kRadialBits>(v[b].x) || too_large<kRadialBits>(v[b].y);
+                seen.add(v[b]);
                 tile[at + slot_of(i + 1)] = pack(lift(v[b]));
             }
         }
     }
-    if (__syncthreads_or(big)) {
+    const unsigned off = block_offset<kRadialBits>(seen);
+    if (off == 0u) {
         const long long base = (long long)(line0 + (active ? q : 0)) * m;
         solve_rho<MODE>(a.psi + base, A.work + base, A.rt, m, active && seg < 2, seg == 0, 1,
                         [](double2 p, int) { return p; });
         return;
+    }
+    if (off != kOff) {
+        if (active)
+            for (int i = seg; i < m; i += lanes) tile[at + slot_of(i + 1)] = pack(lift(row[i], off));
+        __syncthreads();
     }
     const RadLane<MODE> lane(A, coef, active ? seg : (threadIdx.x & 1));
     lane.solve(active, [&](int i) { return unpack(tile[at + slot_of(i)]); },
@@ -825,7 +894,7 @@ __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_rho(const 
 #pragma unroll
         for (int b = 0; b < kIncP; ++b) {
             const int i = seg + b * lanes;
-            if (i < m) row[i] = plus<1, true>(row[i], unpack(tile[at + slot_of(i + 1)]));
+            if (i < m) row[i] = plus<1, true>(row[i], unpack(tile[at + slot_of(i + 1)]), off);
         }
     }
 }
