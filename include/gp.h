@@ -361,10 +361,12 @@ int gp_set_option(gp_ctx *ctx, int option, int value);
 
 /*
  * Autotune the sweep kernels for this context's grid, precision, dt and mode:
- * run `steps` SSCN steps (after one warm-up step) with every eligible (sweep
- * path, tile shape) candidate on the current state, timing each with CUDA
- * events on the context's stream, restore the state after each, and keep
- * the fastest (GP_OPT_SWEEP_PATH / GP_OPT_TILE_SHAPE are set to it).  psi,
+ * run `steps` SSCN steps (after one warm-up step) with GP_PATH_AUTO and every
+ * eligible (sweep path, tile shape) candidate on the current state, timing each
+ * with CUDA events on the context's stream, restore the state after each, and
+ * keep the fastest (GP_OPT_SWEEP_PATH / GP_OPT_TILE_SHAPE are set to it; to
+ * keep a choice, read them).  *path_out names a kernel: where GP_PATH_AUTO won,
+ * the one gp_sweep_paths reports for x.  psi,
  * the pending scale and the step counter are left as they were.  Allocates a
  * temporary copy of psi.  *path_out, *shape_out and *ms_out (mean ms per
  * step of the pick) may be NULL.  Synchronises.

@@ -18,9 +18,9 @@ def cache_path():
                                        "autotune.json"))
 
 
-# Revision of the libraries' tile-shape tables: a cached shape index names an
-# entry of the table it was measured on.
-SHAPE_TABLE = 2
+# Revision of the library's kernels and tile-shape tables: a cached choice
+# holds for the kernels it was measured among, a shape index for its table.
+SHAPE_TABLE = 3
 
 
 def problem_key(shape, h, dt, precision, mode):
@@ -47,7 +47,8 @@ def _store(path, table):
 
 def tune(solver, h, dt, mode, steps=5, path=None):
     """Apply the cached choice for solver's problem class, or autotune and
-    cache it.  Returns the dict {path, shape, ms, cached}."""
+    cache it.  Returns the dict {path, option, shape, ms, cached}: path the
+    kernel, option the GP_OPT_SWEEP_PATH that chooses it."""
     path = path or cache_path()
     key = problem_key(solver.shape, h, dt, solver.precision, mode)
     table = _load(path)
@@ -55,14 +56,15 @@ def tune(solver, h, dt, mode, steps=5, path=None):
     if hit is not None:
         try:
             gp.gp_set_option(solver.ctx, gp.GP_OPT_TILE_SHAPE, hit["shape"])
-            gp.gp_set_option(solver.ctx, gp.GP_OPT_SWEEP_PATH, hit["path"])
+            gp.gp_set_option(solver.ctx, gp.GP_OPT_SWEEP_PATH, hit["option"])
             return dict(hit, cached=True)
-        except gp.GPError:
+        except (gp.GPError, KeyError):
             pass                      # stale entry: tune again
     p, sh, ms = gp.gp_autotune(solver.ctx, steps)
-    table[key] = {"path": p, "shape": sh, "ms": ms}
+    pick = {"path": p, "option": gp.gp_get_option(solver.ctx, gp.GP_OPT_SWEEP_PATH), "shape": sh, "ms": ms}
+    table[key] = pick
     try:
         _store(path, table)
     except OSError:
         pass
-    return {"path": p, "shape": sh, "ms": ms, "cached": False}
+    return dict(pick, cached=False)
