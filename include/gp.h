@@ -68,8 +68,10 @@ enum { GP_IMAG = 0, GP_REAL = 1 };           /* propagation mode            */
 /*
  * psi / sweep precision.  GP_C128: complex128 psi, FP64 arithmetic; where
  * kappa = dt / (4 h^2) is small (<= 0.025 in imaginary, 0.06 in real time) the
- * default path adds to the FP64 psi an increment computed in float-float
- * arithmetic, with a smaller rounding error than FP64 sweeps.  Relative to
+ * sweeps of GP_PATH_AUTO (the default, also of z-slabs and the axial form) and
+ * gp_sweep_noalloc add to the FP64 psi an increment computed in float-float
+ * arithmetic, whose rounding is no larger than an FP64 sweep's (GP_PATH_EXACT
+ * has FP64 arithmetic throughout).  Relative to
  * the largest amplitude of the lines that a block sweeps together, one 2^-30
  * times as large or smaller may carry its increment to 24 bits, one 2^-81
  * times as large or smaller none.
@@ -284,7 +286,8 @@ int gp_slab_observables(gp_ctx *ctx, const double global_sums[9], gp_obs *out);
 
 /* Options of a context (gp_set_option / gp_get_option). */
 enum {
-    /* Sweep kernel: GP_PATH_AUTO picks per axis and mode; GP_PATH_EXACT is a
+    /* Sweep kernel: GP_PATH_AUTO picks per axis and mode; GP_PATH_EXACT
+     * (complex128: FP64 arithmetic, no increments) is a
      * lane pair per line with the elimination scratch in device memory, or,
      * for grids with too few lines to fill the GPU that way, each line in
      * shared memory cut into pieces that many lanes solve at once, starting

@@ -577,7 +577,7 @@ bool axial_inc(const gp_ctx *c, gp::SplitPlan &rho)
     gp::SplitPlan z;
     return c->axial && c->path_opt != GP_PATH_EXACT &&
            gp::rho_inc_plan(c->rt[c->mode], c->grid.nx, c->grid.ny, rho) &&
-           gp::split_plan(c->prec, c->ax[c->mode][1], geom(c->grid, 1), z) && z.increment;
+           gp::split_plan(c->prec, c->ax[c->mode][1], geom(c->grid, 1), z, true) && z.increment;
 }
 
 cudaError_t launch_sweep(gp_ctx *c, int axis, const gp::NonlinArgs *nl, bool nl_at_output,
@@ -606,7 +606,7 @@ cudaError_t launch_sweep(gp_ctx *c, int axis, const gp::NonlinArgs *nl, bool nl_
             fn.scale = nl->scale;
         }
         gp::SplitPlan plan;
-        if (prefers_ff_split(c, axis) && gp::split_plan(GP_C128, ax, g, plan) && plan.increment) {
+        if (prefers_ff_split(c, axis) && gp::split_plan(GP_C128, ax, g, plan, true) && plan.increment) {
             if (blocks) *blocks = gp::split_blocks(plan);
             return gp::launch_sweep_ffinc(plan, c->mode, c->psi, ax, g, nl ? &fn : nullptr, norm, c->stream);
         }
@@ -626,11 +626,13 @@ cudaError_t launch_sweep(gp_ctx *c, int axis, const gp::NonlinArgs *nl, bool nl_
         return gp::launch_sweep_tma(c->prec, c->tile_shape, c->mode, axis, c->maps[axis], ax, g,
                                     nl, norm, c->err_dev, c->stream, nl_at_output);
     }
+    // (a request for the exact path has FP64 arithmetic throughout)
+    const bool fp64_only = c->path_opt == GP_PATH_EXACT;
     if (nl && !nl_at_output)
         return gp::launch_sweep_x(c->prec, c->mode, c->psi, c->work, ax, g, *nl, c->grid.ny,
-                                  c->grid.nz, norm, c->stream);
+                                  c->grid.nz, norm, c->stream, fp64_only);
     return gp::launch_sweep_yz(c->prec, c->mode, c->psi, c->work, ax, g, norm, c->stream,
-                               nl_at_output ? nl : nullptr, blocks);
+                               nl_at_output ? nl : nullptr, blocks, fp64_only);
 }
 
 bool modulated(const gp_ctx *c) { return c->g1 != 0.0; }

@@ -189,7 +189,7 @@ cudaError_t launch_ff_to_c128(void *dst, const void *src, long long count, const
 cudaError_t launch_sweep_x(int prec, int mode, void *psi, void *work,
                            const AxisTables &ax, const SweepGeom &g,
                            const NonlinArgs &nl, int ny, int nz,
-                           const Partials *norm_out, cudaStream_t st);
+                           const Partials *norm_out, cudaStream_t st, bool fp64_only = false);
 // y or z sweep; norm_out != nullptr adds the FP64 sum |u|^2 per block (their
 // number to *blocks, if not null);
 // nlout != nullptr (real time, no norm) applies calcnu to every result
@@ -197,7 +197,8 @@ cudaError_t launch_sweep_x(int prec, int mode, void *psi, void *work,
 cudaError_t launch_sweep_yz(int prec, int mode, void *psi, void *work,
                             const AxisTables &ax, const SweepGeom &g,
                             const Partials *norm_out, cudaStream_t st,
-                            const NonlinArgs *nlout = nullptr, int *blocks = nullptr);
+                            const NonlinArgs *nlout = nullptr, int *blocks = nullptr,
+                            bool fp64_only = false);
 // calcnu as its own pass over every point (x lines; tables in x, y, z order)
 // with the FP64 sums |psi|^2 into `blocks` partials: the imaginary-time
 // symmetric splitting's second half step, after the renormalisation.
@@ -223,15 +224,15 @@ struct SplitPlan {
     bool x = false;              // lines contiguous in memory
     bool after = false;          // programmatic dependent launch (the axis' tables are settled)
     // complex64: the TMA path's arithmetic (else the exact path's); FP64:
-    // float-float increments (sscn_inc.cu; else FP64)
+    // float-float increments (sscn_inc.cu; else FP64 arithmetic)
     bool increment = false;
     int per = 0, threads = 0;    // lines per block, threads per block
     unsigned grid_x = 0, grid_y = 0;
     size_t smem = 0;
 };
-// Whether the sweep of these lines runs that way, and how.
-bool split_plan(int prec, const AxisTables &ax, const SweepGeom &g, SplitPlan &plan,
-                bool increment = false);
+// Whether the sweep of these lines runs that way, and how.  increment: complex64,
+// the TMA path's arithmetic wanted; FP64, float-float increments allowed.
+bool split_plan(int prec, const AxisTables &ax, const SweepGeom &g, SplitPlan &plan, bool increment);
 int split_blocks(const SplitPlan &plan);
 int split_most_blocks(const SweepGeom &g);
 // FP64 psi with float-float increments (sscn_inc.cu): whether kappa allows it,

@@ -643,10 +643,10 @@ int sweep_blocks(const SweepGeom &g)
 cudaError_t launch_sweep_x(int prec, int mode, void *psi, void *work,
                            const AxisTables &ax, const SweepGeom &g,
                            const NonlinArgs &nl, int, int, const Partials *norm_out,
-                           cudaStream_t st)
+                           cudaStream_t st, bool fp64_only)
 {
     SplitPlan plan;
-    if (!norm_out && split_plan(prec, ax, g, plan))
+    if (!norm_out && split_plan(prec, ax, g, plan, prec == kC128 && !fp64_only))
         return launch_sweep_split(plan, prec, mode, psi, ax, g, &nl, false, nullptr, st);
     if (nl.p3) {
         // the precomputed potential factors: FP64 real time, no norm partials
@@ -660,10 +660,10 @@ cudaError_t launch_sweep_x(int prec, int mode, void *psi, void *work,
 cudaError_t launch_sweep_yz(int prec, int mode, void *psi, void *work,
                             const AxisTables &ax, const SweepGeom &g,
                             const Partials *norm_out, cudaStream_t st, const NonlinArgs *nlout,
-                            int *blocks)
+                            int *blocks, bool fp64_only)
 {
     SplitPlan plan;
-    if (!(norm_out && (mode == 1 || g.pstride == 1)) && split_plan(prec, ax, g, plan)) {
+    if (!(norm_out && (mode == 1 || g.pstride == 1)) && split_plan(prec, ax, g, plan, prec == kC128 && !fp64_only)) {
         if (blocks) *blocks = split_blocks(plan);
         return launch_sweep_split(plan, prec, mode, psi, ax, g, nlout, nlout != nullptr, norm_out, st);
     }

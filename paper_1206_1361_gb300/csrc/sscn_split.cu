@@ -482,7 +482,7 @@ bool split_plan(int prec, const AxisTables &ax, const SweepGeom &g, SplitPlan &p
     if (d) {
         // float-float increments where kappa allows them, whatever the number
         // of lines
-        p.increment = inc_applies(ax);
+        p.increment = increment && inc_applies(ax);
         if (p.increment && shape_plan(p, 8, conv, m, d, g)) return true;
         p.increment = false;
     }
