@@ -329,10 +329,11 @@ enum {
 /* GP_PATH_WINDOW (axial form): each line cut into cores solved in parallel,
  * each extended by a window of rows wide enough that the cut coupling reaches
  * the core below 2^-55 (the sweeps then agree with the exact solve to FP64
- * rounding); GP_PATH_AUTO takes it when a line gets at least two cores.  For
- * small dt / (4 h^2) both paths run sweeps in place that cut the lines finer
- * and compute the increment in float-float arithmetic (as GP_C128 does on
- * Cartesian grids). */
+ * rounding); GP_PATH_AUTO takes it when a line gets at least two cores, except
+ * that for small dt / (4 h^2) it runs sweeps in place that cut the lines finer
+ * and compute the increment in float-float arithmetic, as GP_C128 does on
+ * Cartesian grids (gp_sweep_paths reports GP_PATH_WINDOW or GP_PATH_EXACT for
+ * these as well; gp_launches_per_step counts one launch less). */
 /* GP_PATH_SLAB (3D Cartesian grids, nx, ny <= 256, whose xy-plane fits the
  * shared memory of one CTA -- ny (nx | 1) points of 16 (complex128) / 8
  * (complex64) bytes at most 232448 bytes -- or of a 2-CTA cluster, half the

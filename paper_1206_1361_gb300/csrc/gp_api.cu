@@ -566,16 +566,16 @@ bool prefers_ff_split(const gp_ctx *c, int axis)
     return std::max(0.17 * n, p / 150e3) > p / 100e3;
 }
 
-// Axial form: both sweeps with float-float increments, in place, unless the
-// exact path was chosen.  Otherwise the segmented windows (or the exact path)
-// take both.  1024 x 2048 real time, us: 73 + 52 against 175 + 80 in windows; 64 x
+// Axial form: both sweeps with float-float increments, in place, under
+// GP_PATH_AUTO where kappa and the lines' lengths allow.  Otherwise the segmented
+// windows (or the exact path) take both.  1024 x 2048 real time, us: 73 + 52 against 175 + 80 in windows; 64 x
 // 100: 22 against 92 a step.  Imaginary time, 20 steps, 28 grids and dt (both kappa
 // up to 0.0235), relative error against FP64 truth: mean 1.97e-15, rms 1.99e-15, as
 // in windows (1.97e-15, 2.00e-15).
 bool axial_inc(const gp_ctx *c, gp::SplitPlan &rho)
 {
     gp::SplitPlan z;
-    return c->axial && c->path_opt != GP_PATH_EXACT &&
+    return c->axial && c->path_opt == GP_PATH_AUTO &&
            gp::rho_inc_plan(c->rt[c->mode], c->grid.nx, c->grid.ny, rho) &&
            gp::split_plan(c->prec, c->ax[c->mode][1], geom(c->grid, 1), z, true) && z.increment;
 }

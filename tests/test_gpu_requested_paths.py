@@ -37,3 +37,26 @@ def test_the_exact_path_is_not_the_increment_form(shape, mode):
     oracle.step(oracle_params(shape, h, dt, w, g, mode), want, 4)
     assert not np.array_equal(got[gp.GP_PATH_AUTO], got[gp.GP_PATH_EXACT])
     assert all(rel_l2(a, want) <= 1e-12 for a in got.values())
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("mode", [gp.GP_IMAG, gp.GP_REAL])
+def test_axial_windows_run_on_request(mode):
+    """Three launches a step (calcnu, two windowed sweeps) and a norm's finish, where
+    the increment form needs one less."""
+    require_gpu()
+    nr, nz, dt, g = 256, 300, 1e-3, 4.0
+    h = (dt / (4.0 * 0.0125)) ** 0.5
+    psi = rand((nz, nr))
+    psi[1:, 0] = psi[1:, -1]                       # (rho = h / 2 is a live row)
+    got, launches = [], []
+    for path in (gp.GP_PATH_AUTO, gp.GP_PATH_WINDOW, gp.GP_PATH_EXACT):
+        with gp.Solver.axial(nr, nz, h, h, dt, 1.0, 2.0, g, mode) as s:
+            s.set_path(path)
+            got.append(s.load(psi).step(4).psi())
+            launches.append(gp.gp_launches_per_step(s.ctx)[0])
+    par = oracle.AxialParams.make(nr, nz, h, h, dt, 1.0, 2.0, g, mode)
+    want = oracle.axial_step(par, psi.copy(), 4)
+    assert launches[1] == launches[0] + 1
+    assert not np.array_equal(got[0], got[1]) and not np.array_equal(got[0], got[2])
+    assert all(rel_l2(a, want) <= 1e-12 for a in got)
