@@ -1049,6 +1049,18 @@ int materialize(gp_batch *b, gp_batch_slot &s)
     return GP_OK;
 }
 
+// Whether p is memory of the current device, which a kernel may store to; a copy
+// also serves other devices' and reports what it cannot reach.
+bool on_this_device(const void *p)
+{
+    int dev = -1;
+    cudaPointerAttributes at{};
+    if (cudaGetDevice(&dev) == cudaSuccess && cudaPointerGetAttributes(&at, p) == cudaSuccess)
+        return at.type == cudaMemoryTypeDevice && at.device == dev;
+    cudaGetLastError();
+    return false;
+}
+
 template <typename T, int P> cudaError_t launch_tiles(gp_batch *b)
 {
     if (b->args.phase_total[P] == 0) return cudaSuccess;
@@ -1281,7 +1293,7 @@ int gp_batch_store(gp_batch *b, int slot, void *out, int64_t count, int on_devic
     const long long n = (long long)s.grid.nx * s.grid.ny * s.grid.nz;
     if (count != n) return bfail(b, GP_EINVAL, "gp_batch_store: count != nx*ny*nz");
     const size_t align = b->prec == GP_C128 ? 16 : 8;
-    if (on_device && s.scale_pending && reinterpret_cast<uintptr_t>(out) % align == 0) {
+    if (on_device && s.scale_pending && reinterpret_cast<uintptr_t>(out) % align == 0 && on_this_device(out)) {
         // a device buffer takes the scaled psi in the pass that scales it
         const int blocks = (int)std::min<long long>(1024, (n + 255) / 256);
         if (b->prec == GP_C128)
