@@ -936,6 +936,27 @@ int ensure_capacity(gp_batch *b, size_t n_inst)
     return GP_OK;
 }
 
+// Shared memory of the largest tile of any batch (8 lines of 384 complex128, 48.25
+// KB).  A kernel's limit belongs to the function, not to a batch: it is the same
+// for all of them, so that none takes it from another one's launches.
+constexpr int kTileSmem = 64 * 1024;
+
+template <typename T> cudaError_t allow_tiles()
+{
+    cudaError_t e = cudaSuccess;
+    auto allow = [&](auto kern, bool carveout) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmem);
+        if (e == cudaSuccess && carveout)
+            e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                     (int)cudaSharedmemCarveoutMaxShared);
+    };
+    allow(k_batch_steps<T>, false);
+    allow(k_batch_tiles<T, 0>, true);
+    allow(k_batch_tiles<T, 1>, true);
+    allow(k_batch_tiles<T, 2>, true);
+    return e;
+}
+
 // Rebuild the instance descriptors and the item prefix arrays.
 int prepare(gp_batch *b)
 {
@@ -1000,10 +1021,10 @@ int prepare(gp_batch *b)
     GP_BCK(b, cudaGetDevice(&dev));
     GP_BCK(b, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     if (b->prec == GP_C128) {
-        GP_BCK(b, cudaFuncSetAttribute(k_batch_steps<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->smem));
+        GP_BCK(b, allow_tiles<double>());
         GP_BCK(b, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch_steps<double>, 32, b->smem));
     } else {
-        GP_BCK(b, cudaFuncSetAttribute(k_batch_steps<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->smem));
+        GP_BCK(b, allow_tiles<float>());
         GP_BCK(b, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch_steps<float>, 32, b->smem));
     }
     // persistent grid: every resident warp, but no more than the widest
@@ -1064,13 +1085,7 @@ bool on_this_device(const void *p)
 template <typename T, int P> cudaError_t launch_tiles(gp_batch *b)
 {
     if (b->args.phase_total[P] == 0) return cudaSuccess;
-    auto kern = k_batch_tiles<T, P>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                         (int)cudaSharedmemCarveoutMaxShared);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->smem);
-    if (e != cudaSuccess) return e;
-    return gp::launch_after(true, kern, (unsigned)b->args.phase_total[P], 32, b->smem, b->stream, b->args);
+    return gp::launch_after(true, k_batch_tiles<T, P>, (unsigned)b->args.phase_total[P], 32, b->smem, b->stream, b->args);
 }
 
 void stepped(gp_batch *b, int64_t n)
