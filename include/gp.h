@@ -468,7 +468,8 @@ int gp_batch_load(gp_batch *b, int slot, const void *psi, int64_t count, int on_
 int gp_batch_store(gp_batch *b, int slot, void *psi_out, int64_t count, int on_device);
 /* Quench one slot: new g and mode from its next step on. */
 int gp_batch_set_params(gp_batch *b, int slot, double g, int mode);
-/* Advance every instance in the batch by n steps (asynchronous). */
+/* Advance every instance in the batch by n steps.  Asynchronous; beyond some 30000
+ * steps at once the call waits until that many are left to launch. */
 int gp_batch_step(gp_batch *b, int64_t n);
 /*
  * Run the batch's steps as one persistent launch per gp_batch_step from now on,

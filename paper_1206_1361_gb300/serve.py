@@ -15,7 +15,7 @@ A converging solve lowers |dmu| at every check and never meets that rule.
 
 The server admits requests that have arrived, first come first served, as
 long as the batch's memory cap can take their footprint; every instance on the
-device advances together, chunk by chunk, in one persistent launch per chunk;
+device advances together, chunk by chunk, a launch per sweep of a step;
 finished requests leave at a chunk boundary and free their memory, so newly
 arrived ones join while others are mid-solve.  Each instance's arithmetic
 depends only on its own parameters (see gp_batch), so a request's result is
