@@ -182,6 +182,10 @@ int alloc(gp_ctx *c, void **p, size_t bytes)
     return GP_OK;
 }
 
+// Waits for the tables' copies: a copy from pageable memory may return when its
+// source has been staged, and a context's stream does not wait for the legacy one.
+cudaError_t tables_arrived() { return cudaStreamSynchronize(cudaStreamLegacy); }
+
 int upload_tables(gp_ctx *c)
 {
     for (int mode = 0; mode < 2; ++mode) {
@@ -202,7 +206,7 @@ int upload_tables(gp_ctx *c)
             GP_CK(c, cudaMemcpy(d_mult64, mult.data(), m * sizeof(double2), cudaMemcpyHostToDevice));
             GP_CK(c, cudaMemcpy(d_cp32, cp32.data(), m * sizeof(float4), cudaMemcpyHostToDevice));
             GP_CK(c, cudaMemcpy(d_mult32, mult32.data(), m * sizeof(float4), cudaMemcpyHostToDevice));
-            a.settled = true;          // (the copies are synchronous)
+            a.settled = true;          // (create_ctx waits for the copies)
             if (is_ff(c)) {
                 gp::FfAxis &f = c->ffax[mode][k];
                 gp::FfCoef *d_cp = f.cp, *d_mult = f.mult;
@@ -1178,6 +1182,7 @@ int create_ctx(const gp_grid *grid, const double dx[3], double dt, double gamma,
         const double one = 1.0;
         e = cudaMemcpyAsync(c->scale, &one, sizeof(double), cudaMemcpyHostToDevice, c->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+        if (e == cudaSuccess) e = tables_arrived();
         if (e != cudaSuccess) return bail(cuda_fail(c, e, "init"));
     }
     *out = c;
@@ -1798,6 +1803,7 @@ int gp_create_slab(const gp_grid *global, const double dx[3], double dt, double 
     if (!rc) rc = alloc(c, (void **)&c->slab_consts, w.size() * sizeof(double2));
     if (!rc) {
         cudaError_t e = cudaMemcpy(c->slab_consts, w.data(), w.size() * sizeof(double2), cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = tables_arrived();
         if (e != cudaSuccess) rc = cuda_fail(c, e, "gp_create_slab: reduced rows");
     }
     if (!rc) rc = alloc(c, &c->slab_saved, 2 * (size_t)plane * sizeof(double2));
