@@ -351,9 +351,9 @@ def autotune_entry(gp, ctx, case, precision, mode):
 def sweep_rooflines(gp, kt, points, precision, peaks, hbm_peak, hbm_src):
     """Roofline of the dominant sweep of a single-grid step from per-kernel
     times: the arithmetic bound of the float-float form (FP32 lane-operations;
-    measured peak) with the HBM fraction of its algorithmic bytes beside it;
-    for complex128, whose increments run on the FP32 pipe next to a few FP64
-    instructions a point, the HBM fraction."""
+    measured peak), or, for complex128, the FP64 pipe's share of its increment
+    sweeps (their few FP64 instructions a point; the rest of their time is issue
+    slots), with the HBM fraction of its algorithmic bytes beside it."""
     sweeps = {k: v for k, v in kt.items() if k.startswith("sweep") and v > 0}
     dom = max(sweeps, key=sweeps.get)
     bpp = SWEEP_BYTES_PER_POINT[0]
@@ -365,11 +365,11 @@ def sweep_rooflines(gp, kt, points, precision, peaks, hbm_peak, hbm_src):
                     "%.1f T lane-operations/s)" % (peaks["fp32x2_fma"]["tflops"], peak))
         convention = "FP32 lane-operations (add, multiply or fused multiply-add on one lane = 1)"
     else:
-        return {"bound": "hbm", "kernel": dom, "achieved": hbm_achieved, "peak": hbm_peak,
-                "unit": "GB/s", "frac": hbm_achieved / hbm_peak, "peak_source": hbm_src,
-                "bytes_per_point": bpp,
-                "step_hbm_frac": (3 * bpp * points / 1e9) / (sum(sweeps.values()) * 1e-3) / hbm_peak,
-                "kernel_ms": {k: round(v, 5) for k, v in kt.items()}}
+        ops = {k: 8 if k == "sweep_x" else 4 for k in sweeps}
+        peak = peaks["fp64_fma"]["tflops"] / 2
+        peak_src = ("measured FP64 pipe rate (gp_measure_peak, DFMA, %.3f TFLOP/s = %.3f T lane-operations/s)"
+                    % (peaks["fp64_fma"]["tflops"], peak))
+        convention = "FP64 instructions of the increment sweeps a point, on one lane"
     achieved = ops[dom] * points / (sweeps[dom] * 1e-3) / 1e12
     return {"bound": "alu", "kernel": dom, "achieved": achieved, "peak": peak,
             "unit": "TFLOP/s", "frac": achieved / peak, "peak_source": peak_src,
@@ -545,8 +545,8 @@ def run_ours(args):
 def fp64_native_form(gp, torch, stream, case, ground, args, peaks, hbm_peak, hbm_src, ff_value):
     """The same workload on the native FP64 form (complex128 psi, increments in
     float-float arithmetic): the quench from the same ground state, the
-    benchmark's step, its throughput and the HBM fraction of its dominant
-    sweep."""
+    benchmark's step, its throughput and the FP64-pipe and HBM fractions of its
+    dominant sweep."""
     ctx = gp.gp_create(case.shape, case.h, case.dt, *case.trap, case.g, gp.GP_REAL, gp.GP_C128,
                        stream)
     try:

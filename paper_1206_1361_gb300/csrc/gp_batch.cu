@@ -1,7 +1,11 @@
 // gp_batch.cu -- many independent SSCN problems (different grids, traps, g,
-// dt and modes) advanced together by one persistent kernel.
+// dt and modes) advanced together: a launch per sweep of a step over the tiles
+// of every instance (k_batch_tiles), which the stream orders.
 //
-// Work is a queue of items (step s, phase p, instance i, tile t) in that
+// The persistent form (k_batch_steps) runs the same tiles from a queue with
+// bounded waits.  It is slower (below) and stays for gp_batch_set_wait_ns, the
+// interface's failure detection: once a wait budget is set, steps have waits it
+// can bound.  Its work is a queue of items (step s, phase p, instance i, tile t) in that
 // order: phases are the x, y and z Crank-Nicolson sweeps (calclux, calcluy,
 // calcluz; calcnu fused into x) and, in imaginary time, the norm finish
 // (calcnorm).  A tile is 16 or 8 lines of one instance along one axis.  Resident

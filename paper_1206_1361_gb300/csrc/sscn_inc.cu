@@ -11,15 +11,15 @@
 // Here psi stays FP64, but the sweep computes the increment 2 Delta of
 //     (I - kappa L) Delta = kappa L psi,   u = psi + 2 Delta,
 // in float-float arithmetic (sscn_ff.cuh, ~48 significant bits) and adds it to
-// the FP64 psi: 4 FP64 instructions a point (none with drop's MERGE).  |2 Delta| is at most 8 kappa
-// max|psi| and about kappa (k h)^2 |psi| on a smooth state, so with kappa up to
+// the FP64 psi: 4 FP64 instructions a point (2 with drop's MERGE).  |2 Delta| is
+// at most 8 kappa max|psi| and about kappa (k h)^2 |psi| on a smooth state, so with kappa up to
 // kIncKappaReal / kIncKappaImag the rounding of the increment stays at or below
 // that of the FP64 form u = 2 v - psi, which rounds at full size several times.
 // calcnu likewise: the nonlinear factor's distance from 1 is computed in
 // float-float, the potential factor multiplies in FP64.
 //
 // Measured (GB300, 256^3 real time, kappa = 0.0125): y and z sweeps 392 -> 226
-// us, x with calcnu 889 -> 426 us (8 FP64 instructions a point there: 230 us of
+// us, x with calcnu 889 -> 430 us (8 FP64 instructions a point there: 230 us of
 // the FP64 pipe); the y sweep issues about 320 instructions a point, half of
 // them integer conversions and addresses, 62 % of the issue slots, with the FP64
 // pipe 57 % busy (x: 540, 55 % and 53 %).  Relative L2
@@ -29,10 +29,12 @@
 // hardly changes from step to step and the rounding repeats:
 // at kappa = 0.05 (500 x 384, 40 steps) 2.4e-15 against 1.6e-15, hence the
 // smaller kIncKappaImag.  In real time the error moves with kappa through the
-// rounding of the coefficients, the same at every step, in both forms; over
-// kappa = 0.02 .. 0.05, 20 steps, mean and largest, FP64 sweeps and here: 80 x 64
-// x 50 7.3e-15, 2.2e-14 and 5.4e-15, 9.6e-15; 300 x 260 4.7e-15, 8.2e-15 and
-// 3.6e-15, 5.9e-15.
+// rounding of the coefficients, the same at every step, in both forms; 20 steps,
+// mean and largest (e-15), FP64 sweeps and here: kappa 0.004 .. 0.05, 80 x 64 x 50
+// 8.7, 12.9 and 5.7, 7.5; 500 x 384 5.6, 10.0 and 4.8, 8.0; kappa 0.05 .. 0.06 8.1,
+// 18.4 and 7.3, 9.4; 8.1, 16.5 and 5.0, 6.8.  Imaginary time, kappa 0.004 .. 0.025:
+// 2.3, 3.1 and 1.4, 2.0; 1.6, 2.1 and 1.4, 2.0.  (The FP64 truth, dense matrices,
+// has an error of 1.4 to 3e-15 itself: see axial_inc.)
 //
 // The lines are cut and solved as in sscn_split.cu (half sub-lines of at most P
 // rows, whole lines in shared memory).  Per row, r_j = kappa mult_j:

@@ -3,17 +3,18 @@
 // calcluz), the norm reduction (calcnorm) and the observables pass
 // (calcmuen, calcrms) of the paper's "Summary of revisions".
 //
-// Every sweep runs one grid line per thread.  For the y and z sweeps the
-// threads of a warp own neighbouring x, so each load and store of a point is a
-// contiguous warp-wide access; the x sweep walks contiguous lines per thread
-// and leans on L1.  The Thomas elimination is exact: forward elimination
-// writes d'_i to a scratch buffer laid out like psi, back substitution reads
-// it back in reverse.
+// k_sweep gives every line a lane pair.  For the y and z sweeps the lanes of a
+// half warp own neighbouring x, so each load and store of a point is a
+// contiguous access; the x sweep walks contiguous lines per lane and leans on
+// L1.  The elimination is exact: both lanes write d'_i to a scratch buffer
+// laid out like psi and read it back in reverse.  (launch_sweep_x and
+// launch_sweep_yz run the sub-line kernels of sscn_split.cu and sscn_inc.cu
+// where split_plan takes them.)
 //
 // Reductions (norm partials, observables) accumulate in FP64 in a fixed order:
 // per thread sequentially, then a warp-shuffle tree, then per block, so a
-// given launch shape always produces the same bits (the observables do not
-// depend on the launch shape at all: one partials row per grid line).
+// given launch shape always produces the same bits (the observables write a
+// row per block, whose walk follows the grid's shape alone).
 
 #include <algorithm>
 #include <cstdint>
@@ -439,7 +440,7 @@ __global__ void k_add_step(long long *step)
 // terms) sums the differences (the cancellation would amplify FP32 rounding
 // past the 1e-6 the form is held to) with compensated partials per thread.
 //
-// The passes are bound by the FP64 pipe (10 instructions a point at FP64) and,
+// The passes are bound by the FP64 pipe (11 instructions a point at FP64) and,
 // on small grids, by the chain of a thread's walk and of the finish: the walk
 // shortens until there are blocks for every SM, and the finish gives each of
 // the 9 sums a warp of its own.  500 x 384 FP64: 419 us with a thread per whole

@@ -584,7 +584,8 @@ def gp_batch_step(b, n):
 
 
 def gp_batch_set_wait_ns(b, ns):
-    """Budget of each dependency wait of the batch's persistent kernel (ns)."""
+    """Run the batch's steps as one persistent launch from now on, with this
+    budget of each of its dependency waits (ns)."""
     _berr(b, load_library().gp_batch_set_wait_ns(b, int(ns)))
 
 
