@@ -49,13 +49,18 @@
 //
 // Conversions go through the bits of the double with integer instructions (the
 // FP64 <-> FP32 conversion instructions run on the FP64 pipe).  Values enter
-// multiplied by 2^kLift, which puts the full float-float precision at 2^-105
-// .. 2^93.  A block whose largest value lies below 2^-75 (psi is small
-// everywhere, or its lines run far outside the cloud) or above 2^93 lifts it to
-// 2^20 instead; outside 2^-800 .. 2^1000, and with anything not finite, it
-// sweeps in FP64.  So an increment that comes with fewer bits (values below
-// 2^-105) or none (below 2^-156) belongs to a value 2^30 or 2^81 times smaller
-// than the block's largest.
+// multiplied by 2^kLift, which puts the full float-float precision at 2^-165
+// .. 2^33 (|psi| of 10^9, a cloud of a micrometre in metres, lies below).  A
+// block whose largest value lies below 2^-135 (psi is small everywhere, or its
+// lines run far outside the cloud) or above 2^33 lifts it to 2^20 instead;
+// outside 2^-800 .. 2^1000, and with anything not finite, it sweeps in FP64.  So
+// an increment that comes with fewer bits (values below 2^-165) or none (below
+// 2^-216) belongs to a value 2^30 or 2^81 times smaller than the largest of the
+// block.  (Rows of the x sweep that lie in one warp: of the warp.)  On the ground
+// state of the 256^3 quench, whose lines end at 2^-118 and far below, about
+// half of the blocks choose: y 242 us against 227 where psi is nowhere small, x
+// 437 against 433.  A lift of 2^30, with which more did, took 257 and 473 under
+// the profiler.
 
 #include "sscn_ff.cuh"
 #include "sscn_rho.cuh"
@@ -71,7 +76,7 @@ namespace {
 
 constexpr int kIncP = 8;                 // rows a lane
 constexpr double kIncKappaReal = 0.06, kIncKappaImag = 0.025;
-constexpr int kLift = 30;
+constexpr int kLift = 90;
 constexpr int kIncEnds = 2 * kSplitEnds + 1;
 
 struct IncArgs {
@@ -171,24 +176,33 @@ struct Seen {
     __device__ __forceinline__ unsigned value() const { return top == 0u && low != 0u ? 1u : top; }
 };
 
-// The offset of the block's lift, from what its lanes have seen; 0: the block
-// sweeps in FP64.  One barrier where
-// every lane has seen ordinary values or zeros only, three more otherwise.
-template <int MARGIN = 0> __device__ __forceinline__ unsigned block_offset(const Seen &seen)
+// The offset that lifts values up to `top` (a high word; 0: all zero), or 0 where
+// they go to FP64.
+template <int MARGIN> __device__ __forceinline__ unsigned offset_for(unsigned top)
 {
-    constexpr unsigned most = most_of(kOff, MARGIN), tiny = (1023u - 75u) << 20;
+    constexpr unsigned most = most_of(kOff, MARGIN), tiny = (1023u - 45u - kLift) << 20;
     constexpr unsigned least = (1023u - 800u) << 20, huge = (1023u + 1000u) << 20;
-    __shared__ unsigned block_top;
-    unsigned top = seen.value();
-    if (!__syncthreads_or(top != 0u && top - tiny >= most - tiny)) return kOff;
-    if (threadIdx.x == 0) block_top = 0u;
-    __syncthreads();
-    top = __reduce_max_sync(0xffffffffu, top);
-    if ((threadIdx.x & 31) == 0) atomicMax(&block_top, top);
-    __syncthreads();
-    top = block_top;
-    if (top >= tiny && top < most) return kOff;
+    if (top == 0u || (top >= tiny && top < most)) return kOff;
     return top >= least && top < huge ? ((top >> 20) - 127u - 20u) << 20 : 0u;
+}
+
+// The offset of the block's lift, from what its lanes have seen; 0: the block
+// sweeps in FP64.  One barrier where some lane has seen an ordinary value and
+// none a larger one, whatever the others have (a line that ends far outside the
+// cloud); another one otherwise.  block_top: zero before.
+template <int MARGIN = 0> __device__ __forceinline__ unsigned block_offset(const Seen &seen, unsigned *block_top)
+{
+    constexpr unsigned most = most_of(kOff, MARGIN), tiny = (1023u - 45u - kLift) << 20;
+    unsigned top = seen.value();
+    // the barrier counts 1 for a warp with an ordinary value, 31 for one with a larger
+    const bool usual = __any_sync(0xffffffffu, top >= tiny && top < most), large = __any_sync(0xffffffffu, top >= most);
+    const int votes = __syncthreads_count((threadIdx.x & 31) == 0 ? usual : large);
+    static_assert(kSplitThreads / 32 < 31, "the two counts stay apart");
+    if (votes > 0 && votes < 31) return kOff;
+    top = __reduce_max_sync(0xffffffffu, top);
+    if ((threadIdx.x & 31) == 0) atomicMax(block_top, top);
+    __syncthreads();
+    return offset_for<MARGIN>(*block_top);
 }
 
 // ------------------------------------------------------------------ calcnu
@@ -499,6 +513,33 @@ template <int MODE> struct RadLane : HalfLine {
 
 // ----------------------------------------------------------------- kernels
 
+// A lane's points once more, with another lift: i = first, first + step, ... < end of
+// a contiguous row, to row i + shift of the tile; all loads in flight.  (Functions of
+// their own: inlined, they took registers from the kernels, which rarely come here.)
+__noinline__ __device__ void lift_again(const double2 *row, float4 *tile, int first, int step, int end, int shift, unsigned off)
+{
+    double2 v[kIncP];
+#pragma unroll
+    for (int b = 0; b < kIncP; ++b)
+        if (first + b * step < end) v[b] = row[first + b * step];
+#pragma unroll
+    for (int b = 0; b < kIncP; ++b)
+        if (first + b * step < end) tile[slot_of(first + b * step + shift)] = pack(lift(v[b], off));
+}
+
+// The same for the rows row, row + dir, ... row + dir last of a strided line.
+__noinline__ __device__ void lift_again(const double2 *line, long long stride, float4 *tile, int XL, int row, int dir, int last,
+                                        unsigned off)
+{
+    double2 p[kIncP];
+#pragma unroll
+    for (int q = 0; q < kIncP; ++q)
+        if (q <= last) p[q] = line[(row + q * dir) * stride];
+#pragma unroll
+    for (int q = 0; q < kIncP; ++q)
+        if (q <= last) tile[slot_of(row + q * dir) * XL] = pack(lift(p[q], off));
+}
+
 // Resident blocks the kernels are compiled for: 3 of 256 threads (80 registers
 // a thread), or 2 of 512 (64; lines of more than 1024 rows: the z sweep of an
 // axial 1024 x 2048 took 62 us with one, 52 with two).
@@ -513,6 +554,8 @@ __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_x(const __
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ NlScale nl_of_step;
+    __shared__ unsigned block_top;
+    if (threadIdx.x == 0) block_top = 0u;
     const SplitArgs<double> &a = A.s;
     const int n = a.n, pitch = slot_of(n) + 1;
     unsigned char *coef = smem_raw, *coef64 = coef + inc_coef_bytes(a.conv);
@@ -563,13 +606,26 @@ __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_x(const __
                     row[i] = v[b];
                 }
                 seen.add(v[b]);
-                tile[at + slot_of(i)] = pack(lift(v[b]));
             }
         }
     }
     const int own = active ? seg : (threadIdx.x & 1);
-    const unsigned off = block_offset(seen);
-    if (off == 0u) {
+    // rows that lie in one warp each take its lift, without a vote of the block
+    const bool in_warp = 32 % lanes == 0;
+    unsigned off = in_warp ? offset_for<0>(__reduce_max_sync(0xffffffffu, seen.value())) : kOff;
+    if (active) {
+        const unsigned first = off ? off : kOff;
+#pragma unroll
+        for (int b = 0; b < kIncP; ++b)
+            if (1 + seg + b * lanes < n) tile[at + slot_of(1 + seg + b * lanes)] = pack(lift(v[b], first));
+    }
+    bool fp64;
+    if (in_warp) fp64 = __syncthreads_or(off == 0u);
+    else {
+        off = block_offset(seen, &block_top);
+        fp64 = off == 0u;
+    }
+    if (fp64) {
         double2 *t64 = reinterpret_cast<double2 *>(tile);
         stage_coefs<MODE>(a, coef64);
         if (active)
@@ -584,9 +640,8 @@ __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_x(const __
             for (int i = 1 + seg; i < n; i += lanes) row[i] = t64[at + slot_of(i)];
         return;
     }
-    if (off != kOff) {
-        if (active)
-            for (int i = 1 + seg; i < n; i += lanes) tile[at + slot_of(i)] = pack(lift(row[i], off));
+    if (!in_warp && off != kOff) {
+        if (active) lift_again(row, tile + at, 1 + seg, lanes, n, 0, off);
         __syncthreads();
     }
     const IncLane<MODE> lane(A, coef, own);
@@ -614,7 +669,11 @@ __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_yz(const _
     __shared__ double red[32];
     __shared__ NlScale nl_of_step;
     __shared__ volatile unsigned lift_off;
-    if (threadIdx.x == 0) lift_off = kOff;
+    __shared__ unsigned block_top;
+    if (threadIdx.x == 0) {
+        lift_off = kOff;
+        block_top = 0u;
+    }
     const SplitArgs<double> &a = A.s;
     unsigned char *coef = smem_raw, *coef64 = coef + inc_coef_bytes(a.conv);
     float4 *tile = reinterpret_cast<float4 *>(coef64 + coef_bytes<double>(a.conv));
@@ -644,7 +703,7 @@ __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_yz(const _
         if (seg == 0) tile[at_of(0)] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (seg == 1) tile[at_of(n)] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    const unsigned off = block_offset(seen);
+    const unsigned off = block_offset(seen, &block_top);
     Calcnu<double, MODE> nl{};
     const NlScale ns = NLOUT ? nl_of_step : NlScale{};
     if (NLOUT && !P3 && active) nl.setup(a.px, a.py, a.pz, nullptr, nullptr, nullptr, la, lb, 0.0, nullptr);
@@ -677,14 +736,7 @@ __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_yz(const _
     } else {
         if (off != kOff) {
             if (threadIdx.x == 0) lift_off = off;
-            if (active) {
-#pragma unroll
-                for (int q = 0; q < kIncP; ++q)
-                    if (lane.first + q <= lane.last) {
-                        const int i = lane.row(lane.first + q);
-                        tile[at_of(i)] = pack(lift(line[(long long)i * a.pstride], off));
-                    }
-            }
+            if (active) lift_again(line, a.pstride, tile + xl, XL, lane.row(lane.first), lane.top ? 1 : -1, lane.last - lane.first, off);
             __syncthreads();
         }
         lane.template solve<false>(
@@ -828,6 +880,8 @@ __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_rho(const 
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ NlScale nl_of_step;
+    __shared__ unsigned block_top;
+    if (threadIdx.x == 0) block_top = 0u;
     const SplitArgs<double> &a = A.s;
     const int n = a.n, m = n - 1, pitch = slot_of(n) + 1;
     float4 *coef = reinterpret_cast<float4 *>(smem_raw);
@@ -876,7 +930,7 @@ __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_rho(const 
             }
         }
     }
-    const unsigned off = block_offset<kRadialBits>(seen);
+    const unsigned off = block_offset<kRadialBits>(seen, &block_top);
     if (off == 0u) {
         const long long base = (long long)(line0 + (active ? q : 0)) * m;
         solve_rho<MODE>(a.psi + base, A.work + base, A.rt, m, active && seg < 2, seg == 0, 1,
@@ -884,8 +938,7 @@ __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_rho(const 
         return;
     }
     if (off != kOff) {
-        if (active)
-            for (int i = seg; i < m; i += lanes) tile[at + slot_of(i + 1)] = pack(lift(row[i], off));
+        if (active) lift_again(row, tile + at, seg, lanes, m, 1, off);
         __syncthreads();
     }
     const RadLane<MODE> lane(A, coef, active ? seg : (threadIdx.x & 1));
