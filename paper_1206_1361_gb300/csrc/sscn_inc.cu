@@ -19,10 +19,10 @@
 // float-float, the potential factor multiplies in FP64.
 //
 // Measured (GB300, 256^3 real time, kappa = 0.0125): y and z sweeps 392 -> 226
-// us, x with calcnu 889 -> 430 us (8 FP64 instructions a point there: 230 us of
-// the FP64 pipe); the y sweep issues about 320 instructions a point, half of
-// them integer conversions and addresses, 62 % of the issue slots, with the FP64
-// pipe 57 % busy (x: 540, 55 % and 53 %).  Relative L2
+// us, x with calcnu 889 -> 433 us (8 FP64 instructions a point there: 230 us of
+// the FP64 pipe); the y sweep issues about 330 instructions a point, half of
+// them integer conversions and addresses, 63 % of the issue slots, with the FP64
+// pipe 57 % busy (x: 555, 55 % and 53 %).  Relative L2
 // error against FP64 truth, start and here: 64^3 imaginary, 100 steps, 5.3e-15
 // and 2.1e-15; 256^3 real, 10 steps, 6.8e-15 and 4.4e-15; 128 x 96 x 80 real at
 // kappa = 0.05, 20 steps, 1.5e-14 and 6.6e-15.  In imaginary time the state
