@@ -972,7 +972,6 @@ void drop_graph(gp_batch *b)
 int prepare(gp_batch *b)
 {
     if (!b->dirty) return GP_OK;
-    drop_graph(b);
     b->active.clear();
     for (size_t i = 0; i < b->slots.size(); ++i)
         if (b->slots[i].used) b->active.push_back((int)i);
@@ -1016,6 +1015,7 @@ int prepare(gp_batch *b)
     GP_BCK(b, cudaMemcpyAsync(b->d_inst, inst.data(), N * sizeof(Inst), cudaMemcpyHostToDevice, b->stream));
     GP_BCK(b, cudaMemcpyAsync(b->d_ints, ints.data(), ints.size() * sizeof(int), cudaMemcpyHostToDevice, b->stream));
     GP_BCK(b, cudaStreamSynchronize(b->stream));
+    drop_graph(b);                       // (of the batch before; no launch of it is left)
     LaunchArgs &A = b->args;
     A.inst = b->d_inst;
     A.N = N;
