@@ -52,15 +52,18 @@
 // multiplied by 2^kLift, which puts the full float-float precision at 2^-165
 // .. 2^33 (|psi| of 10^9, a cloud of a micrometre in metres, lies below).  A
 // block whose largest value lies below 2^-135 (psi is small everywhere, or its
-// lines run far outside the cloud) or above 2^33 lifts it to 2^20 instead;
-// outside 2^-800 .. 2^1000, and with anything not finite, it sweeps in FP64.  So
+// lines run far outside the cloud) or above 2^33 lifts it to 2^20 instead
+// (below 2^-855 as far as the exponents go); outside 2^-940 .. 2^1000, and with
+// anything not finite, it sweeps in FP64.  So
 // an increment that comes with fewer bits (values below 2^-165) or none (below
 // 2^-216) belongs to a value 2^30 or 2^81 times smaller than the largest of the
 // block.  (Rows of the x sweep that lie in one warp: of the warp.)  On the ground
-// state of the 256^3 quench, whose lines end at 2^-118 and far below, about
-// half of the blocks choose: y 242 us against 227 where psi is nowhere small, x
-// 437 against 433.  A lift of 2^30, with which more did, took 257 and 473 under
-// the profiler.
+// state of the 256^3 quench, whose lines end at 2^-118 and far below, 41 % of
+// the rows choose: y 242 us against 228 where psi is nowhere small, x 441
+// against 436, a step 910 against 876 (with a constant lift 868 on both, and the
+// rows' increments lost).  A usual lift of 2^30, with which more choose, took 257
+// and 473 under the profiler; FP64 from 2^-800 down, which such a state reaches
+// outside its support after a float-float run, 994 a step.
 
 #include "sscn_ff.cuh"
 #include "sscn_rho.cuh"
@@ -176,14 +179,17 @@ struct Seen {
     __device__ __forceinline__ unsigned value() const { return top == 0u && low != 0u ? 1u : top; }
 };
 
+// High words between which some lift reaches full precision.
+constexpr unsigned kLeast = (1023u - 940u) << 20, kHuge = (1023u + 1000u) << 20;
+
 // The offset that lifts values up to `top` (a high word; 0: all zero), or 0 where
-// they go to FP64.
-template <int MARGIN> __device__ __forceinline__ unsigned offset_for(unsigned top)
+// they go to FP64.  ANY: the largest lift there is below kLeast.
+template <int MARGIN, bool ANY = false> __device__ __forceinline__ unsigned offset_for(unsigned top)
 {
     constexpr unsigned most = most_of(kOff, MARGIN), tiny = (1023u - 45u - kLift) << 20;
-    constexpr unsigned least = (1023u - 800u) << 20, huge = (1023u + 1000u) << 20;
     if (top == 0u || (top >= tiny && top < most)) return kOff;
-    return top >= least && top < huge ? ((top >> 20) - 127u - 20u) << 20 : 0u;
+    if ((!ANY && top < kLeast) || top >= kHuge) return 0u;
+    return max((int)(top >> 20) - 127 - 20, 1) << 20;
 }
 
 // The offset of the block's lift, from what its lanes have seen; 0: the block
@@ -610,18 +616,22 @@ __global__ void __launch_bounds__(THREADS, kMinBlocks<THREADS>) k_inc_x(const __
         }
     }
     const int own = active ? seg : (threadIdx.x & 1);
-    // rows that lie in one warp each take its lift, without a vote of the block
+    // rows that lie in one warp each take its lift, without a vote of the block,
+    // which still sweeps in FP64 where all of it is below kLeast
     const bool in_warp = 32 % lanes == 0;
-    unsigned off = in_warp ? offset_for<0>(__reduce_max_sync(0xffffffffu, seen.value())) : kOff;
+    const unsigned top = in_warp ? __reduce_max_sync(0xffffffffu, seen.value()) : 0u;
+    unsigned off = offset_for<0, true>(top);
     if (active) {
-        const unsigned first = off ? off : kOff;
 #pragma unroll
         for (int b = 0; b < kIncP; ++b)
-            if (1 + seg + b * lanes < n) tile[at + slot_of(1 + seg + b * lanes)] = pack(lift(v[b], first));
+            if (1 + seg + b * lanes < n) tile[at + slot_of(1 + seg + b * lanes)] = pack(lift(v[b], off ? off : kOff));
     }
     bool fp64;
-    if (in_warp) fp64 = __syncthreads_or(off == 0u);
-    else {
+    if (in_warp) {
+        // the barrier counts 1 for a warp that a lift serves, 31 for one it does not
+        const int votes = __syncthreads_count((threadIdx.x & 31) == 0 ? top >= kLeast && top < kHuge : top >= kHuge);
+        fp64 = votes >= 31 || (votes == 0 && __syncthreads_or(top != 0u));
+    } else {
         off = block_offset(seen, &block_top);
         fp64 = off == 0u;
     }
