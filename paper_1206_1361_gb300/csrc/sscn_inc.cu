@@ -62,8 +62,8 @@
 // the rows choose: y 242 us against 228 where psi is nowhere small, x 441
 // against 436, a step 910 against 876 (with a constant lift 868 on both, and the
 // rows' increments lost).  A usual lift of 2^30, with which more choose, took 257
-// and 473 under the profiler; FP64 from 2^-800 down, which such a state reaches
-// outside its support after a float-float run, 994 a step.
+// and 473 under the profiler; FP64 from 2^-800 down, which the state of a
+// float-float run reaches outside its support, 995 against 927 a step.
 
 #include "sscn_ff.cuh"
 #include "sscn_rho.cuh"
